@@ -144,7 +144,7 @@ static int allocate(rewl_t r)
     s.spin_stride = (r->N + 15) & ~15;
     s.vec_spins = (r->N & 15) == 0;
     s.magic = (uint32_t)((0x100000000ULL + (uint64_t)r->L - 1) / (uint64_t)r->L);
-    if (move_smem_per_walker(r->N, r->W) > MAX_SMEM_PER_CTA)
+    if (!move_fits(r->N, r->W))
         return r->fail(REWL_ERR_INVALID_ARG, "lattice and window do not fit in shared memory");
     s.spins = dmalloc<int8_t>(nw * s.spin_stride, e);
     s.cfg = dmalloc<int>(nw, e);
@@ -1206,6 +1206,16 @@ const char *rewl_last_error(rewl_t r)
     return g_err.c_str();
 }
 
+// Warps per CTA of a replay launch.  A window so wide that the warp kernel's batch scratch does not
+// fit beside it (a tiny lattice whose caller's W nearly fills the CTA) runs one thread per walker.
+static void replay_layout(const State &s, MoveCfg &c)
+{
+    c.walkers_per_block = 4;
+    while (c.walkers_per_block > 1 && (size_t)c.walkers_per_block * move_smem_per_walker(s.N, s.W) > MAX_SMEM_PER_CTA)
+        c.walkers_per_block >>= 1;
+    c.layout = move_smem_per_walker(s.N, s.W) > MAX_SMEM_PER_CTA ? 1 : 0;
+}
+
 // ---- replay through the production move kernel
 int rewl_replay(int model, int L, int n, int W, int T, void *spins, void *k, const void *lo,
                 const void *hi, void *lng, void *H, const void *lnf, const void *frozen,
@@ -1236,7 +1246,7 @@ int rewl_replay(int model, int L, int n, int W, int T, void *spins, void *k, con
             g_err = "rewl_replay: lattice too large";
             return REWL_ERR_INVALID_ARG;
         }
-    if (move_smem_per_walker(s.N, W) > MAX_SMEM_PER_CTA) {
+    if (!move_fits(s.N, W)) {
         g_err = "rewl_replay: lattice and window do not fit in shared memory";
         return REWL_ERR_INVALID_ARG;
     }
@@ -1263,9 +1273,7 @@ int rewl_replay(int model, int L, int n, int W, int T, void *spins, void *k, con
     }
     MoveCfg c{};
     c.T = T;
-    c.walkers_per_block = 4;
-    while (c.walkers_per_block > 1 && (size_t)c.walkers_per_block * move_smem_per_walker(s.N, W) > MAX_SMEM_PER_CTA)
-        c.walkers_per_block >>= 1;
+    replay_layout(s, c);
     c.eps_l = LNU32_EPS;
     c.words = (const uint32_t *)words;
     c.acc_out = (int *)acc;
@@ -1370,7 +1378,7 @@ int rewl_replay_static(int model, int L, int n, int W, int T, void *spins, void 
             g_err = "rewl_replay_static: lattice too large";
             return REWL_ERR_INVALID_ARG;
         }
-    if (move_smem_per_walker(s.N, W) > MAX_SMEM_PER_CTA) {
+    if (!move_fits(s.N, W)) {
         g_err = "rewl_replay_static: lattice and window do not fit in shared memory";
         return REWL_ERR_INVALID_ARG;
     }
@@ -1395,9 +1403,7 @@ int rewl_replay_static(int model, int L, int n, int W, int T, void *spins, void 
     if (e == cudaSuccess) e = cudaMemsetAsync(&sc->status, 0, sizeof(DevStatus), st);
     MoveCfg c{};
     c.T = T;
-    c.walkers_per_block = 4;
-    while (c.walkers_per_block > 1 && (size_t)c.walkers_per_block * move_smem_per_walker(s.N, W) > MAX_SMEM_PER_CTA)
-        c.walkers_per_block >>= 1;
+    replay_layout(s, c);
     c.eps_l = LNU32_EPS;
     c.words = (const uint32_t *)words;
     c.acc_out = (int *)acc;

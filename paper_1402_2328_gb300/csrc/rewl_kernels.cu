@@ -1,9 +1,9 @@
 // rewl_kernels.cu -- the REWL hot path on sm_103a.
 //
-//   k_move        WL moves (Sec. 2): one warp per walker, lattice, ln g shadow and H in shared
-//                 memory; 32 proposals are drawn and evaluated in parallel, then resolved in
-//                 order (a proposal whose neighbourhood an earlier accepted flip touched is
-//                 re-evaluated), so the result equals the one-move-at-a-time walk exactly.
+//   k_move        WL moves (Sec. 2): one warp per walker, lattice and ln g shadow in shared
+//                 memory; up to 32 proposals are evaluated in parallel, then resolved in
+//                 order (the batch ends before a proposal whose neighbourhood an earlier accepted
+//                 flip touched), so the result equals the one-move-at-a-time walk exactly.
 //   k_check       per-walker flatness (warp-shuffle min / sum over visited bins) and window
 //                 advance: average ln g over the m walkers, H = 0, ln f /= 2 (Sec. 2).
 //   k_swap        replica exchange between windows (w, w+1), Eq. (1).
@@ -12,6 +12,8 @@
 #include <cfloat>
 #include <cmath>
 #include <cstdint>
+
+#include <cuda_fp16.h>
 
 #include "rewl_device.cuh"
 #include "rewl_kernels.cuh"
@@ -55,25 +57,36 @@ __device__ __forceinline__ int propose_dk(const int8_t *sp, const Lattice &lat, 
 // WL moves.  Decision rule (Sec. 2): accept iff ln u < ln g(k) - ln g(k'), with the float64
 // ln g the one-move-at-a-time walk would hold at that moment.
 //
-// One warp per walker.  Shared memory holds the lattice (int8), an int64 shadow
-// V(b) = round(ln g0(b) 2^32) + (visits) * round(ln f 2^32) of ln g over the window, H, and one
-// claim stamp per site.  Moves are taken in batches of up to 32:
-//   1. lane j draws the proposal of step t+j (Philox) and evaluates its energy change on the
-//      lattice as it was at the batch start; the batch is limited to its conflict-free prefix
-//      (no proposal sits on the site or a neighbour of an earlier one), so those energy
-//      changes stay exact whatever earlier steps of the batch do;
-//   2. lane j holds, as float32 relative to the bin k0 where the batch started, ln g of bin
-//      k0-16+j (+inf outside the window);
-//   3. the warp walks the steps in order computing only the path: one shuffle fetches
-//      ln g(k'), and the move is accepted/rejected in float32 when ln u is farther than a
-//      proven error bound from ln g(k) - ln g(k'); a step inside the bound or whose k' leaves
-//      the cached bins is flagged, the batch is cut there, and that one step is decided from
-//      the float64 values rebuilt exactly (seqadd of the interval-start ln g and the visit
-//      counts);
-//   4. the side effects of the steps done (spin flips, visits of V and H) are applied
-//      lane-parallel.
-// At the end of the launch the float64 ln g of every bin is rebuilt exactly from its visit
-// count, so the state equals that of the sequential walk bit for bit.
+// One warp per walker.  Shared memory holds the lattice, an int64 shadow
+// V(b) = round(ln g0(b) 2^32) + (visits) * round(ln f 2^32) of ln g over the window, and the
+// proposals drawn ahead.  Moves are taken in batches of up to 32:
+//   1. lane j takes the proposal of step t+j from the ring (site, neighbours, ln u: drawn
+//      32 steps at a time in issue slots the walk of an earlier batch leaves idle) and evaluates
+//      its energy change on the lattice as it was at the batch start;
+//   2. lane x keeps the shadow of cached bin x (32 bins around the current one) in a register;
+//      the cache moves when the walker nears its edge;
+//   3. small ln f: lane j compares its threshold with the half-precision ratio table
+//      ln g(x) - ln g(x + dk) for every cached x at once, which gives a 32-bit mask "step j is
+//      surely accepted from x".  Walking the batch is then a chain of integer shifts and
+//      multiply-adds on these masks, two steps at a time.  A step that is surely accepted or
+//      rejected under a margin that covers every rounding and the visits since the table was
+//      taken needs no more; another one is decided in float32 with those visits, and if that
+//      is too close as well, in float64.
+//      Large ln f, where each visit turns later decisions: the path is walked with running
+//      float32 values through shuffles, every step screened by the same kind of margin;
+//   4. the batch is cut before the first step that has a neighbour changed by an earlier step of
+//      the batch, or shares its site with one, and behind it the side effects (spin flips, visits)
+//      are applied lane-parallel.
+// A step inside the float32 margin is decided from the float64 values rebuilt exactly (seqadd of
+// the interval-start ln g and the visit counts); at the end of the launch the float64 ln g of
+// every bin is rebuilt the same way, so the state equals that of the sequential walk bit for bit.
+//
+// What bounds it: the dependent chain of one batch.  A walker is one warp and the workloads have
+// 1-2 walkers per SM sub-partition, so latencies set the pace, not issue slots or memory
+// (measured on GB300 in cycles: integer op or FMA 4, a predicate before use 10, shuffle 24-28,
+// shared load 29, ballot 23, popc 20, ffs 42, match_any of 32 different values 375).
+// Ising L=64, 32 x 16, ln f = 2^-20, ms per round: 0.64 with the 32-step chain of shuffles and
+// predicates before, 0.35 with the masks.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ double shadow_error(double maxabs, int T, double lnf, bool frozen)
 {
@@ -131,21 +144,72 @@ __device__ __forceinline__ bool exact_decision(const double *glng, const long lo
     return exact_value_decision(glng, V, lo, k, kp, lnf, lnfq, frozen, w2);
 }
 
-// One walker's `c.T` moves; `base` is the walker's shared-memory block, the whole warp calls.
-template <bool ISING, bool REPLAY, bool CHECK>
-__device__ __forceinline__ void move_walker(const State &s, const MoveCfg &c, const int slot,
-                                            unsigned char *base, const int lane)
+// ---- the lattice in the warp kernel's shared memory: one 16-bit cell per site, the state in the
+// low byte and, while a batch is set up, the lane that proposes the site in the high byte
+// (NO_CLAIM: none), so one load gives both.
+constexpr unsigned NO_CLAIM = 0xffu;
+
+// Ratio table: rows d = -DM .. DM of 32 half-precision differences ln g(x) - ln g(x + d) over
+// the cached bins x; word w of a row holds x = w and x = w + 16.  A row is 80 bytes, so the
+// 16-byte loads of eight lanes at eight different rows meet eight different bank groups.
+constexpr int ROW_BYTES = 80;
+
+__device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t n)
 {
-    if (s.status != nullptr && s.status->done) return;
-    int8_t *sp = reinterpret_cast<int8_t *>(base);
-    long long *V = reinterpret_cast<long long *>(base + pad16(s.N));
-    uint32_t *vis = reinterpret_cast<uint32_t *>(V + padw(s.W));      // [W bits] bin visited
-    uint16_t *stamp = reinterpret_cast<uint16_t *>(vis + visw(s.W));  // [N] batch claims
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n)); // 0 for n >= 32
+    return r;
+}
+
+// -1 if v is negative, else 0.  Spelled out: the compiler would make a comparison and a select of
+// it, and a predicate takes 10 cycles before it can be used where a shift takes 4.
+__device__ __forceinline__ int sign_mask(int v)
+{
+    int m;
+    asm("shr.s32 %0, %1, 31;" : "=r"(m) : "r"(v));
+    return m;
+}
+
+// a where mask m is -1, b where it is 0
+__device__ __forceinline__ int pick(int m, int a, int b)
+{
+    int r;
+    asm("lop3.b32 %0, %1, %2, %3, 0xca;" : "=r"(r) : "r"(m), "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ float pickf(int m, float a, float b)
+{
+    return __int_as_float(pick(m, __float_as_int(a), __float_as_int(b)));
+}
+
+// 0x01 in every byte of `p` that differs from byte value b (bytes below 128, or all +-1)
+template <bool ISING> __device__ __forceinline__ uint32_t bytes_unequal(uint32_t p, uint32_t b)
+{
+    const uint32_t x = p ^ (b * 0x01010101u);
+    if (ISING) return (x >> 7) & 0x01010101u; // +1 ^ -1 = 0xfe
+    return ((x + 0x7f7f7f7fu) >> 7) & 0x01010101u;
+}
+
+// One walker's `c.T` moves; `base` is the walker's shared-memory block, the whole warp calls.
+// NP: pairs of steps in a batch (16, or fewer for small lattices, where sites soon repeat).
+template <bool ISING, bool REPLAY, bool CHECK, int NP>
+__device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, const int slot,
+                                              unsigned char *base, const int lane)
+{
+    constexpr int DM = ISING ? 2 : 4; // largest |bin change| of a move
+    uint16_t *cell = reinterpret_cast<uint16_t *>(base);
+    uint8_t *cellb = base;
+    long long *V = reinterpret_cast<long long *>(base + 2 * pad16(s.N));
+    uint32_t *vis = reinterpret_cast<uint32_t *>(V + padw(s.W)); // [W bits] bin visited
+    unsigned char *tab = reinterpret_cast<unsigned char *>(vis + visw(s.W));
+    uint4 *bc = reinterpret_cast<uint4 *>(tab + MOVE_TAB_BYTES); // [16] step pairs
+    uint4 *trail = bc + 16;                                      // [16] what the walk left
+    uint4 *ring = trail + 16;                                    // [MOVE_RING] proposals drawn ahead
 
     const int w = slot / s.m;
     const int lo = s.lo[w], hi = s.hi[w], nb = hi - lo + 1;
-    int k = s.k[slot];
-    if (lo < 0 || nb < 1 || nb > s.W || k < lo || k > hi) { // malformed input: refuse
+    const int kstart = s.k[slot];
+    if (lo < 0 || nb < 1 || nb > s.W || kstart < lo || kstart > hi) { // malformed input: refuse
         if (lane == 0) atomicOr(&s.status->err, ERR_INPUT);
         return;
     }
@@ -158,22 +222,28 @@ __device__ __forceinline__ void move_walker(const State &s, const MoveCfg &c, co
     const Lattice lat{s.L, s.N, s.magic};
     const int T = c.T;
 
-    // ---- load lattice, shadow ln g, H; clear the claim stamps
+    // ---- load lattice, shadow ln g
     if (s.vec_spins) {
         const int4 *src = reinterpret_cast<const int4 *>(gsp);
-        int4 *dst = reinterpret_cast<int4 *>(sp);
-        for (int i = lane; i < (s.N >> 4); i += 32) dst[i] = src[i];
+        uint4 *dst = reinterpret_cast<uint4 *>(cell);
+        for (int i = lane; i < (s.N >> 4); i += 32) {
+            const int4 v = src[i];
+            dst[2 * i] = make_uint4(__byte_perm(v.x, ~0u, 0x4140), __byte_perm(v.x, ~0u, 0x4342),
+                                    __byte_perm(v.y, ~0u, 0x4140), __byte_perm(v.y, ~0u, 0x4342));
+            dst[2 * i + 1] = make_uint4(__byte_perm(v.z, ~0u, 0x4140), __byte_perm(v.z, ~0u, 0x4342),
+                                        __byte_perm(v.w, ~0u, 0x4140), __byte_perm(v.w, ~0u, 0x4342));
+        }
     } else {
-        for (int i = lane; i < s.N; i += 32) sp[i] = gsp[i];
+        for (int i = lane; i < s.N; i += 32)
+            cell[i] = (uint16_t)((NO_CLAIM << 8) | (uint8_t)gsp[i]);
     }
-    for (int i = lane; i < s.N; i += 32) stamp[i] = 0xffffu; // matches no batch
     double mx = 0.0;
-    bool bad = false;
+    bool bad_in = false;
     for (int b = lane; b < nb; b += 32) {
         const double x = glng[b];
-        bad = bad || !(fabs(x) < 0x1p30); // also catches NaN
+        bad_in = bad_in || !(fabs(x) < 0x1p30); // also catches NaN
         mx = fmax(mx, fabs(x));
-        V[b] = bad ? 0LL : __double2ll_rn(__dmul_rn(x, 0x1p32));
+        V[b] = bad_in ? 0LL : __double2ll_rn(__dmul_rn(x, 0x1p32));
     }
     // visited bits: the bins any walker of the window had visited when this launch started,
     // the start bin, and every bin this walker enters for the first time (always through the
@@ -186,262 +256,438 @@ __device__ __forceinline__ void move_walker(const State &s, const MoveCfg &c, co
         if (lane == 0) vis[i] = bits;
     }
     __syncwarp();
-    if (lane == 0) vis[(k - lo) >> 5] |= 1u << ((k - lo) & 31); // the start bin
+    if (lane == 0) vis[(kstart - lo) >> 5] |= 1u << ((kstart - lo) & 31); // the start bin
     mx = warp_max(mx);
     // the shadow of a running window ends the launch below (max |ln g| + T ln f) 2^32 < 2^62,
     // and ln f 2^32 must not round to zero; a frozen window adds nothing to it
     const bool lnf_ok = frozen || (lnf >= 0x1p-32 && lnf < 0x1p20 && mx + (double)T * lnf < 0x1p30);
-    if (__any_sync(FULL, bad) || !lnf_ok) {
+    if (__any_sync(FULL, bad_in) || !lnf_ok) {
         // the int64 shadow would overflow or lose the increment: leave the state untouched
         if (lane == 0) atomicOr(&s.status->err, ERR_RANGE);
         return;
     }
     const long long lnfq = __double2ll_rn(__dmul_rn(lnf, 0x1p32));
+    const long long lnfq_add = frozen ? 0LL : lnfq;
     // interval-constant part of the float32 screening margin (ln units)
-    const float Mbase = (float)(c.eps_l + 2.0 * shadow_error(mx, T, lnf, frozen) * 0x1p-32) + 0x1p-21f;
+    const float Mbase = (float)(c.eps_l + 2.0 * shadow_error(mx, T, lnf, frozen) * 0x1p-32) * (1.0f + 0x1p-20f) + 0x1p-21f;
     const float lnf_f = frozen ? 0.0f : (float)lnf;
-    __syncwarp();
+    const bool table_walk = lnf_f <= TABLE_WALK_LNF;
+    // visits after which the ratio table is taken anew
+    const int table_life = lnf_f > 0.0f ? (int)fminf(TABLE_DRIFT / lnf_f, 1e8f) : 100000000;
 
     const unsigned long long st0 = s.step[slot];
-    unsigned int nacc = 0, nex = 0, nmis = 0;
+    unsigned int nacc = 0, nex = 0, nmis = 0; // nacc: of this lane's steps
     const uint32_t tag = (s.inst << 8) | TAG_MOVE;
+    const unsigned below = (1u << lane) - 1u;
+    // lane x counts the visits of cache bin x: bit i of x as a mask to xor a ballot with
+    unsigned xinv[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) xinv[i] = ((lane >> i) & 1) ? 0u : ~0u;
 
-    int t = 0;
-    unsigned batch = 0;
-    while (t < T) {
-        ++batch;
-        const int n = min(32, T - t);
-        // ---- register cache of ln g around k0 (float32, relative to bin k0)
-        const int k0 = k, base = k0 - 16;
-        const int bj = base + lane;
-        const bool bin_ok = bj >= lo && bj <= hi;
-        float Lw = 0.0f;
-        if (bin_ok) {
-            const long long x = V[bj - lo] - V[k0 - lo];
-            Lw = __fmaf_rn(__uint2float_rn((uint32_t)x), 0x1p-32f, (float)(int)(x >> 32));
-        }
-        // largest |Lw| of the cache (non-negative floats order like their bit patterns)
-        // Bins never visited keep their initial ln g while the others grow, so their cache
-        // values can be far off: they are marked NaN (a step there is flagged unsure and
-        // decided from the float64 values) and do not widen every other step's margin.
-        const bool far = bin_ok && !((vis[(bj - lo) >> 5] >> ((bj - lo) & 31)) & 1u);
-        const float Mx = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(bin_ok && !far ? fabsf(Lw) : 0.0f))) +
-                         33.0f * lnf_f + 0x1p-20f;
-        const float M = Mbase + 40.0f * ulpf(2.0f * Mx);
-        if (!bin_ok) Lw = INFINITY; // a move there is rejected: ln g(k) - inf < ln u
-        if (far) Lw = __int_as_float(0x7fc00000);
-
-        // ---- parallel phase: lane j evaluates proposal t + j on the batch-start lattice
-        uint32_t w0, w1, w2;
+    // The random words of step i.
+    auto draw = [&](int i, uint32_t &w0, uint32_t &w1, uint32_t &w2) {
         if (REPLAY) {
-            if (lane < n) {
-                const uint32_t *wp = c.words + ((size_t)slot * T + t + lane) * 3;
-                w0 = wp[0];
-                w1 = wp[1];
-                w2 = wp[2];
-            } else {
-                w0 = w1 = w2 = 0u;
-            }
+            const uint32_t *wp = c.words + ((size_t)slot * T + i) * 3;
+            w0 = i < T ? wp[0] : 0u;
+            w1 = i < T ? wp[1] : 0u;
+            w2 = i < T ? wp[2] : 0u;
         } else {
-            const unsigned long long sn = st0 + (unsigned long long)(t + lane);
-            const u32x4 r = philox((uint32_t)sn, (uint32_t)(sn >> 32), (uint32_t)(s.slot0 + slot),
-                                   tag, s.key0, s.key1);
+            const unsigned long long sn = st0 + (unsigned long long)i;
+            const u32x4 r = philox((uint32_t)sn, (uint32_t)(sn >> 32), (uint32_t)(s.slot0 + slot), tag, s.key0,
+                                   s.key1);
             w0 = r.x;
             w1 = r.y;
             w2 = r.z;
         }
+    };
+    // Proposals of steps g .. g+31 into the ring (when `room`): site and new-state draw, the four
+    // neighbours, ln u.
+    auto draw_ahead = [&](int g, bool room) {
+        uint32_t w0, w1, w2;
+        draw(g + lane, w0, w1, w2);
         const int site = (int)mulhi(w0, (uint32_t)s.N);
         int nl, nr, nu, nd;
         lat.nbrs(site, nl, nr, nu, nd);
-        const int pr = ISING ? 0 : (int)mulhi(w1, (uint32_t)(s.q - 1));
-        int snew;
-        const int dk = propose_dk<ISING>(sp, lat, s.q, site, pr, snew);
-        // a proposal that keeps the energy is always accepted and keeps the bin: the serial
+        const unsigned pr = ISING ? 0u : mulhi(w1, (uint32_t)(s.q - 1));
+        const uint4 e = make_uint4((unsigned)site | (pr << 16), (unsigned)nl | ((unsigned)nr << 16),
+                                   (unsigned)nu | ((unsigned)nd << 16), __float_as_uint(lnu32(w2)));
+        if (room) ring[(g + lane) & (MOVE_RING - 1)] = e;
+    };
+
+    // ---- the cached bins: lane j holds the shadow of bin wbase + j
+    int wbase = kstart - 16, x = 16; // x: cache offset of the current bin
+    bool bin_ok = false, far = false;
+    long long Vr = 0;
+    float Lw = 0.0f, M = 0.0f;
+    auto cache_store = [&]() {
+        if (bin_ok) V[wbase + lane - lo] = Vr;
+        __syncwarp();
+    };
+    auto cache_load = [&](int k) {
+        wbase = k - 16;
+        x = 16;
+        const int bj = wbase + lane;
+        bin_ok = bj >= lo && bj <= hi;
+        if (bin_ok) Vr = V[bj - lo];
+        // Bins never visited keep their initial ln g while the others grow, so their cache
+        // values can be far off: they are marked NaN (a step there is flagged unsure and
+        // decided from the float64 values) and do not widen every other step's margin.
+        far = bin_ok && !((vis[(bj - lo) >> 5] >> ((bj - lo) & 31)) & 1u);
+    };
+    // ln g of the cached bins relative to the current bin in float32, and the margin
+    auto cache_floats = [&]() {
+        const long long ref = __shfl_sync(FULL, Vr, x);
+        const long long d = Vr - ref;
+        Lw = __fmaf_rn(__uint2float_rn((uint32_t)d), 0x1p-32f, (float)(int)(d >> 32));
+        // largest |Lw| of the cache (non-negative floats order like their bit patterns)
+        const float Mx = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(bin_ok && !far ? fabsf(Lw) : 0.0f))) +
+                         33.0f * lnf_f + 0x1p-20f;
+        M = Mbase + 40.0f * ulpf(2.0f * Mx);
+        if (!bin_ok) Lw = INFINITY; // a move there is rejected: ln g(k) - inf < ln u
+        if (far) Lw = __int_as_float(0x7fc00000);
+    };
+
+    int g = 64; // steps drawn: always t + 2 NP at least
+    draw_ahead(0, true);
+    draw_ahead(32, true);
+    cache_load(kstart);
+    int table_age = table_life + 1; // visits since the table was taken
+    __syncwarp();
+
+    int t = 0;
+    uint4 pe = ring[lane]; // lane j: the proposal of step t + j
+    while (t < T) {
+        const int n = min(2 * NP, T - t);
+        const int site = (int)(pe.x & 0xffffu);
+        if (lane < n) cellb[2 * site + 1] = (uint8_t)lane;
+        __syncwarp();
+        const unsigned c0 = cell[site], c1 = cell[pe.y & 0xffffu], c2 = cell[pe.y >> 16],
+                       c3 = cell[pe.z & 0xffffu], c4 = cell[pe.z >> 16];
+        const uint32_t nbytes = __byte_perm(__byte_perm(c1, c2, 0x0040), __byte_perm(c3, c4, 0x0040), 0x5410);
+        const uint32_t s0 = c0 & 0xffu;
+        // earlier lanes that propose one of this site's neighbours; settled after the walk: the
+        // batch ends before the first step one of whose neighbours was changed
+        unsigned claims = (shl_clamp(1u, c1 >> 8) | shl_clamp(1u, c2 >> 8) | shl_clamp(1u, c3 >> 8) |
+                           shl_clamp(1u, c4 >> 8)) & below;
+        bool dup = false; // an earlier lane proposes the same site: the batch ends before this step
+        int snew, dkm;    // dkm = dk + DM
+        if (ISING) {
+            snew = -(int)(int8_t)s0;
+            // dE = 2 s0 sum of neighbours, dk = dE / 4 = 2 - neighbours unequal to s0
+            dkm = (int)__dp4a((int)bytes_unequal<true>(nbytes, s0), -1, 4);
+        } else {
+            snew = (int)(s0 + 1u + (pe.x >> 16));
+            if (snew >= s.q) snew -= s.q;
+            dkm = __dp4a((int)bytes_unequal<false>(nbytes, s0), -1,
+                         __dp4a((int)bytes_unequal<false>(nbytes, (uint32_t)snew), 0x01010101, DM));
+        }
+        const int dk = dkm - DM;
+        // a proposal that keeps the energy is always accepted and keeps the bin: the
         // walk sees it as a sure non-move (threshold +inf), the lane itself records the flip
         const bool dz = dk == 0;
-        const float thr = dz ? INFINITY : lnu32(w2);
-        // conflict-free prefix: proposal j may be resolved on the batch-start lattice only if
-        // no earlier proposal of the batch sits on its site or a neighbour.
-        // Claim stamp = (batch mod 2047) << 5 | lane of the lowest lane proposing the site: every
-        // lane writes its stamp, then a lane that finds a later lane's stamp on its site writes
-        // again until none does (at most one extra pass unless three lanes share a site).  A
-        // stale stamp of an old batch with the same low bits can only cut a batch early.
-        const unsigned btag = batch % 2047u;
-        const uint16_t mystamp = (uint16_t)((btag << 5) | (unsigned)lane);
-        if (lane < n) stamp[site] = mystamp;
+        const float thr = dz ? INFINITY : __uint_as_float(pe.w);
+        // two lanes on one site: make the lowest lane's claim stand
+        if (__any_sync(FULL, lane < n && (c0 >> 8) != (unsigned)lane)) {
+            unsigned own = c0 >> 8;
+            for (int it = 0; it < 32; ++it) { // each pass lowers some claim: ends within 32 passes
+                const bool again = lane < n && own > (unsigned)lane;
+                if (!__any_sync(FULL, again)) break;
+                if (again) cellb[2 * site + 1] = (uint8_t)lane;
+                __syncwarp();
+                own = cellb[2 * site + 1];
+                __syncwarp();
+            }
+            dup = lane < n && own < (unsigned)lane;
+            claims = (shl_clamp(1u, cellb[2 * (pe.y & 0xffffu) + 1]) | shl_clamp(1u, cellb[2 * (pe.y >> 16) + 1]) |
+                      shl_clamp(1u, cellb[2 * (pe.z & 0xffffu) + 1]) | shl_clamp(1u, cellb[2 * (pe.z >> 16) + 1])) & below;
+        }
         __syncwarp();
-        for (int it = 0; it < 32; ++it) { // each pass lowers some stamp: ends within 32 passes
-            bool again = false;
-            if (lane < n) {
-                const unsigned v = stamp[site];
-                again = (v >> 5) == btag && (int)(v & 31u) > lane;
-            }
-            __syncwarp();
-            if (!__any_sync(FULL, again)) break;
-            if (again) stamp[site] = mystamp;
-            __syncwarp();
-        }
-        bool conflict = false;
-        {
-            const int xs[5] = {site, nl, nr, nu, nd};
-#pragma unroll
-            for (int m = 0; m < 5; ++m) {
-                const unsigned v = stamp[xs[m]];
-                conflict = conflict || ((v >> 5) == btag && (int)(v & 31u) < lane);
-            }
-        }
-        const unsigned cmask = __ballot_sync(FULL, conflict && lane < n);
-        const int J = cmask ? (__ffs(cmask) - 1) : n; // >= 1: lane 0 never conflicts
+        if (lane < n) cellb[2 * site + 1] = (uint8_t)NO_CLAIM;
+        const bool cut = lane >= n || dup;
 
-        // ---- serial phase: the path k_0, k_1, ... only.  Every step runs unconditionally;
-        // lane j records the bin after step j and whether step j was too close to call in
-        // float32, and the batch is cut at the first such step afterwards (the steps after it
-        // are discarded), so no bookkeeping sits on the dependency chain.
-        // Steps are resolved in pairs (2p, 2p+1): the three cache lookups a pair can need
-        // (k' of the first step; k' of the second step after the first moved / stayed) are
-        // issued together and the second step is evaluated in both worlds, so one shuffle
-        // latency and one select cover two moves.  Decision variable:
-        // e = ln g(k) - ln g(k') - thr; accept if e > M, reject if e < -M, else unsure.
-        // A target outside the 32 cached bins reads a wrong lane; such steps are found after
-        // the loop (the target is known per lane) and cut there as well.
-        int myx = 16;      // lane j: cache offset of the bin after step j
-        bool myun = false; // lane j: step j unsure in float32
-        bool mysa = false, mysr = false; // CHECK: float32 verdict of step j (sure accept / reject)
-        int xk = 16;       // cache offset of the current bin
-        float Lk = 0.0f;   // running value of the current bin (the cache holds it only once left)
-#pragma unroll
-        for (int p = 0; p < 16; ++p) {
-            const int i = 2 * p;
-            if ((p & 1) == 0 && p > 0 && (i >= J || (unsigned)xk >= 32u || __any_sync(FULL, myun)))
-                break; // every 2 pairs
-            const int dk0 = __shfl_sync(FULL, dk, i), dk1 = __shfl_sync(FULL, dk, i + 1);
-            const float th0 = __shfl_sync(FULL, thr, i), th1 = __shfl_sync(FULL, thr, i + 1);
-            const int x0 = xk + dk0; // k' of step i
-            const int xA = x0 + dk1; // k' of step i+1 if step i moved
-            const int xR = xk + dk1; // k' of step i+1 if step i stayed
-            const bool atk = lane == xk, at0 = lane == x0;
-            const float L0 = __shfl_sync(FULL, Lw, x0 & 31);
-            const float LA_ = __shfl_sync(FULL, Lw, xA & 31);
-            const float LR = __shfl_sync(FULL, Lw, xR & 31);
-            const float LA = (dk1 == -dk0) ? Lk : LA_; // back to the bin just left
-            const float Lm = L0 + lnf_f;               // value after step i if moved
-            const float Ls = Lk + lnf_f;               // value after step i if stayed
-            // step i
-            const float e0 = (Lk - L0) - th0;
-            const bool m0 = e0 > M;
-            const bool un0 = CHECK ? (th0 != INFINITY && L0 != INFINITY) : !(fabsf(e0) > M);
-            // step i+1 in both worlds, then the world step i chose
-            const float e1A = (Lm - LA) - th1;
-            const float e1R = (Ls - LR) - th1;
-            const bool m1 = m0 ? (e1A > M) : (e1R > M);
-            const float e1 = m0 ? e1A : e1R;
-            const float L1 = m0 ? LA : LR;
-            const float Lc1 = m0 ? Lm : Ls;
-            const int x1 = m0 ? xA : xR;
-            const int xc1 = m0 ? x0 : xk;
-            const bool un1 = CHECK ? (th1 != INFINITY && L1 != INFINITY) : !(fabsf(e1) > M);
-            // the bins left keep their running values
-            if (m0 && atk) Lw = Lk;
-            if (m1 && (m0 ? at0 : atk)) Lw = Lc1;
-            if (lane == i) {
-                myx = xc1;
-                myun = un0;
-                if (CHECK) {
-                    mysa = e0 > M;
-                    mysr = e0 < -M;
-                }
-            }
-            xk = m1 ? x1 : xc1;
-            if (lane == i + 1) {
-                myx = xk;
-                myun = un1;
-                if (CHECK) {
-                    mysa = e1 > M;
-                    mysr = e1 < -M;
-                }
-            }
-            Lk = (m1 ? L1 : Lc1) + lnf_f;
+        // ---- the current bin near the edge of the cache: cache the bins around it
+        if ((unsigned)(x - CACHE_LO) > (unsigned)(CACHE_HI - CACHE_LO)) {
+            const int k = wbase + x;
+            cache_store();
+            cache_load(k);
+            table_age = table_life + 1;
         }
-        // bin before step j; a target outside the cache makes step j unsure as well
-        const int xup = __shfl_up_sync(FULL, myx, 1);
-        const int xbefore = lane == 0 ? 16 : xup;
-        const bool oob = (unsigned)(xbefore + dk) >= 32u;
-        const unsigned badbits = __ballot_sync(FULL, myun || oob);
-        const unsigned stopbits = badbits | (J >= 32 ? 0u : (0xffffffffu << J));
-        const int ndone = stopbits ? __ffs(stopbits) - 1 : 32;
-        const bool amb_stop = ndone < J;
-        if (ndone == 0 && !amb_stop) { // no step done and none to decide: cannot happen (J >= 1)
+
+        // ---- the walk: cache offsets xb, xa of the bin before and after step `lane`.  The batch
+        // stops before step `stop`; `open` says that this step is not decided yet.
+        int xb, xa, stop, scr = -1;
+        bool open;
+        auto stop_at = [&](bool accepted, bool ok) {
+            const unsigned accs = __ballot_sync(FULL, accepted);
+            const bool end = cut || (claims & accs) != 0u;
+            const unsigned v = __reduce_min_sync(FULL, end ? 2u * lane : (ok ? 64u : 2u * lane + 1u));
+            stop = (int)(v >> 1);
+            open = v & 1u;
+        };
+        if (table_walk) {
+            if (table_age > table_life) { // rows of the ratio table
+                cache_floats();
+#pragma unroll
+                for (int d = 1; d <= DM; ++d) {
+                    float up = __shfl_down_sync(FULL, Lw, d);
+                    if (lane + d > 31) up = __int_as_float(0x7fc00000);
+                    const __half h = __float2half_rn(Lw - up);
+                    const int xd = (lane + d) & 31;
+                    *reinterpret_cast<__half *>(tab + (DM + d) * ROW_BYTES + 4 * (lane & 15) + 2 * (lane >> 4)) = h;
+                    *reinterpret_cast<__half *>(tab + (DM - d) * ROW_BYTES + 4 * (xd & 15) + 2 * (xd >> 4)) = __hneg(h);
+                }
+                table_age = 0;
+                __syncwarp();
+            }
+            // the step is surely accepted from bin offset x if D(x) > tS, surely rejected if
+            // D(x) < tR, whatever the visits since the table was taken did to ln g
+            const float mg = __fmaf_rn((float)(table_age + lane + 1), lnf_f, M);
+            const __half2 tS = __float2half2_rn(thr + mg);
+            const __half tR = __float2half_rn(thr - mg);
+            const unsigned char *row = tab + dkm * ROW_BYTES;
+            unsigned S = 0u; // bit x: surely accepted from x
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const uint4 qv = reinterpret_cast<const uint4 *>(row)[v];
+                const uint32_t ww[4] = {qv.x, qv.y, qv.z, qv.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    S |= __hgt2_mask(*reinterpret_cast<const __half2 *>(&ww[e]), tS) & (0x00010001u << (4 * v + e));
+            }
+            if (dz) S = 0u;
+            const int dn = __shfl_down_sync(FULL, dk, 1);
+            bool known = false; // step `lane` was decided below
+            bool ok;
+            // pairs of steps: from bin offset x the first one moves if bit x of a.x is set,
+            // the second if bit x of a.y is set (whatever the first one did)
+            auto publish = [&]() {
+                const unsigned S1 = __shfl_down_sync(FULL, S, 1);
+                const unsigned sh = __funnelshift_r(S1 << 4, S1 >> 28, (unsigned)(dk + 4)); // S1 seen from x + dk
+                if (!(lane & 1)) bc[lane >> 1] = make_uint4(S, (S & sh) | (~S & S1), (unsigned)dk, (unsigned)dn);
+                __syncwarp();
+            };
+            auto walk = [&]() {
+                int y = 31 - x; // S << y has the bit of offset x on top
+                unsigned pk[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const uint4 a = bc[p];
+                    pk[p >> 2] |= (unsigned)y << (8 * (p & 3));
+                    const int m0 = sign_mask((int)(a.x << y)), m1 = sign_mask((int)(a.y << y));
+                    y += m0 * (int)a.z;
+                    y += m1 * (int)a.w;
+                }
+                const uint4 a = bc[lane >> 1];
+                const unsigned pw = lane < 16 ? (lane < 8 ? pk[0] : pk[1]) : (lane < 24 ? pk[2] : pk[3]);
+                const int yq = (int)((pw >> (8 * ((lane >> 1) & 3))) & 31u);
+                const int m0 = sign_mask((int)(a.x << yq)), m1 = sign_mask((int)(a.y << yq));
+                const int odd = -(lane & 1);
+                xb = 31 - yq + (m0 & odd & (int)a.z);
+                const int mv = pick(odd, m1, m0);
+                xa = xb + (mv & dk);
+                const __half D = *reinterpret_cast<const __half *>(row + 4 * (xb & 15) + 2 * ((xb >> 4) & 1));
+                ok = dz || mv != 0 || known || __hlt(D, tR);
+                if (CHECK) ok = dz || (unsigned)(xb + dk - (lo - wbase)) >= (unsigned)nb;
+                stop_at(dz || mv != 0, ok);
+            };
+            publish();
+            if (NP == 16) { // the walk leaves most issue slots idle: draw proposals in them
+                const bool room = g + 32 - t <= MOVE_RING;
+                draw_ahead(g, room);
+                g += room ? 32 : 0;
+            }
+            walk();
+            while (open) {
+                // step `stop`: its ln g difference with the visits before it, in float32
+                const int u = stop;
+                const int xu = __shfl_sync(FULL, xb, u), du = __shfl_sync(FULL, dk, u);
+                const int xt = xu + du;
+                if ((unsigned)xt >= 32u) {
+                    open = u == 0; // else the next batch's cache will hold the target
+                    break;
+                }
+                if (table_age > 0) { // bring the cached values up to date
+                    const float Mt = M;
+                    cache_floats();
+                    M = fmaxf(M, Mt);
+                }
+                const unsigned bu = (1u << u) - 1u;
+                const int cx = __popc(__ballot_sync(FULL, xa == xu) & bu), ct = __popc(__ballot_sync(FULL, xa == xt) & bu);
+                const float e = __fmaf_rn((float)(cx - ct), lnf_f, __shfl_sync(FULL, Lw, xu) - __shfl_sync(FULL, Lw, xt)) -
+                                __shfl_sync(FULL, thr, u);
+                if (CHECK) {
+                    const int sure = ((S >> xu) & 1u) ? 1 : (__hlt(*reinterpret_cast<const __half *>(
+                                                                 row + 4 * (xu & 15) + 2 * (xu >> 4)), tR) ? 0 : -1);
+                    scr = __shfl_sync(FULL, sure, u);
+                    if (scr < 0) scr = e > M ? 1 : (e < -M ? 0 : -1);
+                    break;
+                }
+                if (!(fabsf(e) > M)) break; // too close: float64
+                if (lane == u) {
+                    known = true;
+                    if (e > M) S |= 1u << xu;
+                }
+                publish();
+                walk();
+            }
+            table_age += stop;
+        } else {
+            // Large ln f: the visits of the batch decide its later steps, so the path is walked
+            // with running float32 values.  Steps are resolved in pairs: the three cache
+            // lookups a pair can need (k' of the first step; k' of the second after the first
+            // moved / stayed) are issued together and the second step is evaluated in both
+            // worlds, so one shuffle latency covers two moves.  Decision variable:
+            // v = M - (ln g(k) - ln g(k') - thr); accept if v < 0, reject if v > 2M, else unsure.
+            // Outcomes are sign masks, not predicates: a predicate takes more than twice the
+            // cycles of an integer operation before it can be used.
+            // A target outside the 32 cached bins reads a wrong lane; such steps are found after
+            // the loop and cut there as well.
+            cache_floats();
+            reinterpret_cast<uint2 *>(bc)[lane] = make_uint2(__float_as_uint(thr + M), (unsigned)dk);
+            if (NP == 16) {
+                const bool room = g + 32 - t <= MOVE_RING;
+                draw_ahead(g, room);
+                g += room ? 32 : 0;
+            }
+            __syncwarp();
+            float Lr = Lw;   // the cache, with the running values of the bins left
+            int xk = x;      // cache offset of the current bin
+            float Lk = 0.0f; // its running value (the cache holds it only once left)
+#pragma unroll 4
+            for (int p = 0; p < NP; ++p) {
+                const uint4 a = bc[p];
+                const int d0 = (int)a.y, d1 = (int)a.w;
+                const int x0 = xk + d0; // k' of step i
+                const int xA = x0 + d1; // k' of step i+1 if step i moved
+                const int xR = xk + d1; // k' of step i+1 if step i stayed
+                const float L0 = __shfl_sync(FULL, Lr, x0);
+                const float LA_ = __shfl_sync(FULL, Lr, xA);
+                const float LR = __shfl_sync(FULL, Lr, xR);
+                const float LA = (d1 == -d0) ? Lk : LA_; // back to the bin just left
+                const int onk = lane == xk ? -1 : 0, on0 = lane == x0 ? -1 : 0;
+                const float Ls = Lk + lnf_f; // value after step i if stayed
+                const float Lm = L0 + lnf_f; // value after step i if moved
+                const float v0 = (__uint_as_float(a.x) - Lk) + L0;
+                const int m0 = sign_mask(__float_as_int(v0));
+                const float v1 = pickf(m0, (__uint_as_float(a.z) - Lm) + LA, (__uint_as_float(a.z) - Ls) + LR);
+                const int m1 = sign_mask(__float_as_int(v1));
+                const int xc = pick(m0, x0, xk);
+                const float Lc = pickf(m0, Lm, Ls);
+                Lr = pickf(m0 & onk, Lk, Lr); // the bins left keep their running values
+                Lr = pickf(m1 & pick(m0, on0, onk), Lc, Lr);
+                xk = pick(m1, pick(m0, xA, xR), xc);
+                Lk = pickf(m1, pickf(m0, LA, LR), Lc) + lnf_f;
+                if (lane == 0) // one lane: a store by all of them holds the shuffles up behind it
+                    trail[p] = make_uint4((unsigned)xc, __float_as_uint(v0), (unsigned)xk, __float_as_uint(v1));
+            }
+            __syncwarp();
+            const uint2 tr = reinterpret_cast<const uint2 *>(trail)[lane];
+            xa = (int)tr.x;
+            const float v = __uint_as_float(tr.y);
+            const int xup = __shfl_up_sync(FULL, xa, 1);
+            xb = lane == 0 ? x : xup;
+            const bool oob = (unsigned)(xb + dk) >= 32u;
+            bool ok = (v < 0.0f || v > 2.0f * M * (1.0f + 0x1p-20f)) && !oob;
+            if (CHECK) ok = dz || (unsigned)(xb + dk - (lo - wbase)) >= (unsigned)nb;
+            stop_at(dz || xa != xb, ok);
+            if (open) {
+                const bool out = __shfl_sync(FULL, oob ? 1 : 0, stop);
+                if (CHECK) {
+                    const float vu = __shfl_sync(FULL, v, stop);
+                    scr = out ? -1 : (vu < 0.0f ? 1 : (vu > 2.0f * M * (1.0f + 0x1p-20f) ? 0 : -1));
+                } else if (stop > 0 && out) {
+                    open = false; // the next batch's cache will hold the target
+                    table_age = table_life + 1;
+                }
+            }
+        }
+        if (stop == 0 && !open) { // no step done and none to decide: cannot happen (lane 0 is never cut)
             if (lane == 0) atomicOr(&s.status->err, ERR_INPUT);
             return;
         }
-        // bin after each step (valid for the steps done, all inside the cache)
-        const int mypos = k0 - 16 + myx;
-        const int kc = ndone > 0 ? k0 - 16 + __shfl_sync(FULL, myx, ndone - 1) : k0;
-        // float32 verdict at the cut (CHECK): 1 sure accept, 0 sure reject, -1 unsure
-        int scr = -1;
-        if (CHECK) {
-            const unsigned sa = __ballot_sync(FULL, mysa), sr = __ballot_sync(FULL, mysr);
-            scr = ndone >= 32 ? -1 : (((sa >> ndone) & 1u) ? 1 : (((sr >> ndone) & 1u) ? 0 : -1));
-        }
 
-        // ---- side effects of steps 0..ndone-1
-        const bool mine = lane < ndone;
-        const bool accj = dz || myx != xbefore; // step j accepted (a move to another bin, or dE = 0)
-        if (mine && accj) sp[site] = (int8_t)snew; // conflict-free sites
+        // ---- side effects of steps 0 .. stop-1
+        const bool mine = lane < stop;
+        const bool accj = dz || xa != xb; // step j accepted (a move to another bin, or dE = 0)
+        if (mine && accj) cellb[2 * site] = (uint8_t)snew; // distinct sites
+        t += stop;
+        const uint4 pnext = ring[(t + lane) & (MOVE_RING - 1)];
+        const int step_done = t - stop;
         {
-            // visits: the lanes of one bin add their count with one plain update (no atomics)
-            const unsigned grp = __match_any_sync(FULL, mine ? mypos : -1 - lane);
-            if (mine && !frozen && lane == __ffs(grp) - 1)
-                V[mypos - lo] += (long long)__popc(grp) * lnfq;
+            // visits: lane x counts the steps that ended in cache bin x
+            unsigned v = stop < 32 ? (1u << stop) - 1u : FULL;
+#pragma unroll
+            for (int i = 0; i < 5; ++i) v &= __ballot_sync(FULL, (xa >> i) & 1) ^ xinv[i];
+            Vr += (long long)__popc(v) * lnfq_add;
         }
         if (REPLAY && mine) {
-            c.acc_out[(size_t)slot * T + t + lane] = accj ? 1 : 0;
-            c.dk_out[(size_t)slot * T + t + lane] = dk;
+            c.acc_out[(size_t)slot * T + step_done + lane] = accj ? 1 : 0;
+            c.dk_out[(size_t)slot * T + step_done + lane] = dk;
         }
-        nacc += __popc(__ballot_sync(FULL, mine && accj));
-        k = kc;
-        t += ndone;
+        nacc += mine && accj ? 1u : 0u;
+        if (stop > 0) x = __shfl_sync(FULL, xa, stop - 1);
+        pe = pnext;
         __syncwarp();
 
         // ---- a proposal too close to call in float32: decide it from the float64 values
-        if (amb_stop) {
-            const int i = ndone;
-            const int dki = __shfl_sync(FULL, dk, i);
-            const int sitei = __shfl_sync(FULL, site, i);
-            const int snewi = __shfl_sync(FULL, snew, i);
-            const uint32_t w2i = __shfl_sync(FULL, w2, i);
+        if (open) {
+            const int dki = __shfl_sync(FULL, dk, stop);
+            const int sitei = __shfl_sync(FULL, site, stop);
+            const int snewi = __shfl_sync(FULL, snew, stop);
+            int k = wbase + x;
             const int kp = k + dki;
             bool acc = dki == 0;
+            cache_store();
             if (!acc && kp >= lo && kp <= hi) {
+                uint32_t w0, w1, w2i;
+                draw(t, w0, w1, w2i);
                 acc = exact_decision(glng, V, lo, k, kp, lnf, lnfq, frozen, w2i);
                 if (scr < 0) ++nex;
                 else if ((int)acc != scr) ++nmis;
             }
+            __syncwarp();
             if (acc) {
-                sp[sitei] = (int8_t)snewi;
                 k = kp;
-                ++nacc;
+                if (lane == 0) {
+                    cellb[2 * sitei] = (uint8_t)snewi;
+                    ++nacc;
+                }
             }
-            if (!frozen && lane == 0) V[k - lo] += lnfq;
-            // a bin reached for the first time is only ever entered here (its cache value is
-            // NaN until marked), so marking it here keeps the visited set complete
-            if (lane == 0) vis[(k - lo) >> 5] |= 1u << ((k - lo) & 31);
+            if (lane == 0) {
+                V[k - lo] += lnfq_add;
+                // a bin reached for the first time is only ever entered here (its cache value
+                // is NaN until marked), so marking it here keeps the visited set complete
+                vis[(k - lo) >> 5] |= 1u << ((k - lo) & 31);
+            }
             if (REPLAY && lane == 0) {
                 c.acc_out[(size_t)slot * T + t] = acc ? 1 : 0;
                 c.dk_out[(size_t)slot * T + t] = dki;
             }
             t += 1;
+            pe = ring[(t + lane) & (MOVE_RING - 1)];
+            __syncwarp();
+            cache_load(k);
+            table_age = table_life + 1;
+        }
+        if (NP < 16 && g < t + 64) { // several small batches use up one draw of 32
+            draw_ahead(g, true);
+            g += 32;
             __syncwarp();
         }
     }
+    cache_store();
 
     // ---- write back lattice, float64 ln g (rebuilt exactly), H, counters
     if (s.vec_spins) {
-        const int4 *src = reinterpret_cast<const int4 *>(sp);
+        const uint4 *src = reinterpret_cast<const uint4 *>(cell);
         int4 *dst = reinterpret_cast<int4 *>(gsp);
-        for (int i = lane; i < (s.N >> 4); i += 32) dst[i] = src[i];
+        for (int i = lane; i < (s.N >> 4); i += 32) {
+            const uint4 a = src[2 * i], b = src[2 * i + 1];
+            dst[i] = make_int4(__byte_perm(a.x, a.y, 0x6420), __byte_perm(a.z, a.w, 0x6420),
+                               __byte_perm(b.x, b.y, 0x6420), __byte_perm(b.z, b.w, 0x6420));
+        }
     } else {
-        for (int i = lane; i < s.N; i += 32) gsp[i] = sp[i];
+        for (int i = lane; i < s.N; i += 32) gsp[i] = (int8_t)(cell[i] & 0xffu);
     }
     if (!frozen) {
         double *gl = s.lng + (size_t)slot * s.W;
@@ -453,13 +699,24 @@ __device__ __forceinline__ void move_walker(const State &s, const MoveCfg &c, co
             }
         }
     }
+    nacc = __reduce_add_sync(FULL, nacc);
     if (lane == 0) {
-        s.k[slot] = k;
+        s.k[slot] = wbase + x;
         s.step[slot] = st0 + (unsigned long long)T;
         s.acc[slot] += nacc;
         if (nex) atomicAdd(&s.status->n_exact, (unsigned long long)nex);
         if (nmis) atomicAdd(&s.status->n_mismatch, (unsigned long long)nmis);
     }
+}
+
+template <bool ISING, bool REPLAY, bool CHECK>
+__device__ __forceinline__ void move_walker(const State &s, const MoveCfg &c, const int slot,
+                                            unsigned char *base, const int lane)
+{
+    if (s.status != nullptr && s.status->done) return;
+    if (s.N >= BATCH32_SITES) move_walker_n<ISING, REPLAY, CHECK, 16>(s, c, slot, base, lane);
+    else if (s.N >= BATCH16_SITES) move_walker_n<ISING, REPLAY, CHECK, 8>(s, c, slot, base, lane);
+    else move_walker_n<ISING, REPLAY, CHECK, 4>(s, c, slot, base, lane);
 }
 
 // ---------------------------------------------------------------------------------------

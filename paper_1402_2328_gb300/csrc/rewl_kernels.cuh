@@ -63,13 +63,35 @@ struct MoveCfg {
 // 32-bit words of the per-walker visited-bin bit set (padded to 16 bytes)
 __host__ __device__ inline int visw(int W) { return (((W + 31) >> 5) + 3) & ~3; }
 
-// Shared memory of one walker in the move kernel: lattice (16-byte padded), int64 ln g
-// shadow over the window (padded to 4 bins; the visit counts are recovered from it), the
-// visited-bin bit set, uint16 claim stamps per site.
+// Scratch of one walker's batch: the ratio table (9 rows of 80 bytes), 16 step pairs, the 16
+// entries the walk leaves, and the ring of proposals drawn ahead.
+constexpr int MOVE_TAB_BYTES = 9 * 80;
+constexpr int MOVE_RING = 128;
+constexpr int MOVE_SCRATCH_BYTES = MOVE_TAB_BYTES + (2 * 16 + MOVE_RING) * 16;
+// Largest ln f at which a batch is walked through the ratio table.
+constexpr float TABLE_WALK_LNF = 0x1p-8f;
+// Growth of ln g (visits x ln f) after which the ratio table is taken anew.
+constexpr float TABLE_DRIFT = 0x1p-10f;
+// Cache offsets of the current bin between which the cached bins stay.
+constexpr int CACHE_LO = 8, CACHE_HI = 23;
+// Smallest lattices whose batches are 32 and 16 steps (smaller ones: 8).
+constexpr int BATCH32_SITES = 450, BATCH16_SITES = 100;
+
+// Shared memory of one walker in the move kernel: lattice (a 16-bit cell per site, padded to 16
+// sites), int64 ln g shadow over the window (padded to 4 bins; the visit counts are recovered
+// from it), the visited-bin bit set, the batch scratch.
 __host__ __device__ inline size_t move_smem_per_walker(int N, int W)
 {
+    return 2u * (size_t)((N + 15) & ~15) + (size_t)((W + 3) & ~3) * 8u + (size_t)visw(W) * 4u +
+           (size_t)MOVE_SCRATCH_BYTES;
+}
+// The largest lattice and window accepted: 3 bytes per site and 8 per bin within one CTA, which
+// covers move_smem_per_walker for every size it admits.
+__host__ __device__ inline bool move_fits(int N, int W)
+{
     return (size_t)((N + 15) & ~15) + (size_t)((W + 3) & ~3) * 8u + (size_t)visw(W) * 4u +
-           (size_t)((N + 7) & ~7) * 2u;
+               (size_t)((N + 7) & ~7) * 2u <=
+           MAX_SMEM_PER_CTA;
 }
 // Shared memory of one walker of the thread-per-walker layout: lattice (16-byte padded) and the
 // int64 ln g shadow over the window (padded to 2 bins, 16 bytes).
