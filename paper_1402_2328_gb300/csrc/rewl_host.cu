@@ -431,17 +431,21 @@ int rewl_init(rewl_t r)
         lohi[w] = r->lo[w];
         lohi[h + w] = r->hi[w];
     }
-    // per-walker initial ln g (0, or the warm start)
-    std::vector<double> lng(h * r->m * W, 0.0);
-    if (!r->lng_init.empty())
+    // per-walker initial ln g: 0, or the warm start
+    std::vector<double> lng;
+    if (!r->lng_init.empty()) {
+        lng.assign(h * r->m * W, 0.0);
         for (size_t w = 0; w < h; ++w)
             for (int i = 0; i < r->m; ++i)
                 for (int b = r->lo[w]; b <= r->hi[w]; ++b)
                     lng[(w * r->m + i) * W + (b - r->lo[w])] = r->lng_init[b];
+    }
     std::vector<double> lnf(h, r->lnf_init);
     std::vector<uint8_t> fin(h, (uint8_t)(r->lnf_init < r->lnf_final));
     e = cudaMemcpyAsync(r->d_lohi, lohi.data(), lohi.size() * sizeof(int), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s.lng, lng.data(), lng.size() * 8, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+        e = lng.empty() ? cudaMemsetAsync(s.lng, 0, h * r->m * W * 8, st)
+                        : cudaMemcpyAsync(s.lng, lng.data(), lng.size() * 8, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(s.lnf, lnf.data(), h * 8, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(s.finished, fin.data(), h, cudaMemcpyHostToDevice, st);
     const size_t nw = (size_t)r->nw;

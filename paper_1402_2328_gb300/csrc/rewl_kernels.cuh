@@ -93,6 +93,8 @@ __host__ __device__ inline bool move_fits(int N, int W)
                (size_t)((N + 7) & ~7) * 2u <=
            MAX_SMEM_PER_CTA;
 }
+// Shared memory of one walker in the prep kernel: a 16-bit cell per site.
+__host__ __device__ inline size_t prep_smem_per_walker(int N) { return 2u * (size_t)((N + 15) & ~15); }
 // Shared memory of one walker of the thread-per-walker layout: lattice (16-byte padded) and the
 // int64 ln g shadow over the window (padded to 2 bins, 16 bytes).
 __host__ __device__ inline size_t move_smem_per_thread_walker(int N, int W)

@@ -69,3 +69,30 @@ def test_replay_of_rows_that_fill_shared_memory(call):
     assert np.array_equal(kd.cpu().numpy(), st["k"])
     assert np.array_equal(lg.cpu().numpy()[:, :12].view(np.uint64), st["lng"].view(np.uint64))
     assert np.array_equal(Hd.cpu().numpy().view(np.uint32)[:, :12], st["H"])
+
+
+# windows narrower than one move's largest step, so that the prep walk can jump over them; a
+# budget that ends inside a batch
+@pytest.mark.parametrize("model,L,width,budget", [(0, 6, 3, 100), (3, 6, 3, 100), (10, 8, 2, 100),
+                                                  (10, 13, 40, 1), (0, 13, 30, 1)])
+def test_prep_bit_exact(model, L, width, budget):
+    import paper_1402_2328_gb300.rewl as R
+    B = O.num_bins(model, L)
+    lo = np.arange(0, B - width + 1, max(1, width - 1), dtype=np.int32)
+    hi = (lo + width).astype(np.int32)
+    hi[-1] = B
+    args = (model, L, len(lo), 0.75, 3, 1e-4, 0.8)
+    seed = I.seed_for(8, L + model)
+    g = R.REWL(model, L, 1, 0.75, 3, 1e-4, 0.8, seed=seed, prep_budget=budget)
+    g.set_windows(lo, hi)
+    o = O.REWL(*args, seed=seed, lo_hi=(lo, hi), prep_budget=budget)
+    try:
+        g.init()
+        failed = False
+    except R.REWLError:
+        failed = True  # some window out of reach: the walkers' states still agree
+    assert (o.init() != 0) == failed
+    gs, os_ = {f: g.get_state(f) for f in ("spins", "k", "pstep", "prep_restarts")}, o.state()
+    for f in gs:
+        assert np.array_equal(gs[f], os_[f]), f
+    g.close()
