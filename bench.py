@@ -192,7 +192,7 @@ def workload_config(args, wl, world):
             "l2": "flushed (256 MB write) before every timed step"}
 
 
-KERNEL_SOURCES = ["paper_1402_2328_gb300/csrc/rewl_kernels.cu",
+KERNEL_SOURCES = ["paper_1402_2328_gb300/csrc/rewl_move.cuh",
                   "paper_1402_2328_gb300/csrc/rewl_kernels.cuh",
                   "paper_1402_2328_gb300/csrc/rewl_device.cuh"]
 

@@ -11,7 +11,9 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "librewl.so")
-SOURCES = ["rewl_kernels.cu", "rewl_host.cu", "rewl_batch.cu", "rewl_mlp.cu", "rewl_em.cu"]
+SOURCES = ["rewl_kernels.cu", "rewl_move_ising.cu", "rewl_move_potts.cu", "rewl_move_replay.cu",
+           "rewl_move_check.cu", "rewl_move_batch.cu", "rewl_move_batch_ahead.cu",
+           "rewl_move_batch_check.cu", "rewl_host.cu", "rewl_batch.cu", "rewl_mlp.cu", "rewl_em.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",
          "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",

@@ -147,6 +147,13 @@ static cudaError_t enqueue_batch_round(rewl_batch_t b)
     c.T = (int)b->interval;
     c.walkers_per_block = b->block_walkers;
     c.check_all = b->check_all;
+    long long walkers = 0;
+    size_t per = 1;
+    for (rewl_t r : b->inst) {
+        walkers += r->nw;
+        per = std::max(per, move_smem_per_walker(r->N, r->W));
+    }
+    c.ahead = b->thread_sites == 0 && draw_ahead_pays(walkers, b->sms, b->block_walkers, per);
     c.eps_l = LNU32_EPS;
     cudaError_t e = cudaSuccess;
     std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
@@ -161,7 +168,7 @@ static cudaError_t enqueue_batch_round(rewl_batch_t b)
         if (e == cudaSuccess) e = cudaEventRecord(ev.first, b->stream);
     }
     if (e == cudaSuccess)
-        e = launch_move_batch(b->d_states, b->d_jobs, b->njobs, b->block_walkers, b->smem, c, b->stream);
+        e = launch_move_batch(b->d_states, b->d_jobs, b->njobs, b->smem, c, b->stream);
     if (b->profile && e == cudaSuccess) {
         e = cudaEventRecord(ev.second, b->stream);
         b->ev_used.push_back(ev);

@@ -481,6 +481,7 @@ cudaError_t rewl_enqueue_round(rewl_t r)
     c.layout = r->layout;
     c.walkers_per_block = r->layout ? thread_walkers_per_block(r) : walkers_per_block(r);
     c.check_all = r->check_all;
+    c.ahead = draw_ahead_pays(r->nw, r->sms, c.walkers_per_block, move_smem_per_walker(r->N, r->W));
     c.eps_l = LNU32_EPS;
     cudaError_t e = cudaSuccess;
     std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};

@@ -14,7 +14,7 @@ struct DevStatus {
     unsigned long long n_exact;   // moves decided by the float64 path
     unsigned long long n_mismatch;// check_all: screen decisions that disagreed (must stay 0)
 };
-enum : int { ERR_PREP = 1, ERR_RANGE = 2, ERR_INPUT = 4 };
+enum : int { ERR_PREP = 1, ERR_RANGE = 2, ERR_INPUT = 4, ERR_STALL = 8 };
 constexpr int MAX_M = 1024; // walkers per window (exchange permutation in shared memory)
 constexpr size_t MAX_SMEM_PER_CTA = 227u * 1024u;
 
@@ -55,6 +55,7 @@ struct MoveCfg {
     int walkers_per_block;  // walkers per CTA (warps, or threads with layout 1)
     int layout;             // 0: one warp per walker, 1: one thread per walker
     int check_all;
+    int ahead;              // a second warp per walker draws its proposals
     double eps_l;
     const uint32_t *words;  // replay: [nw][T][3], else nullptr (Philox)
     int *acc_out, *dk_out;  // replay: [nw][T]
@@ -63,27 +64,41 @@ struct MoveCfg {
 // 32-bit words of the per-walker visited-bin bit set (padded to 16 bytes)
 __host__ __device__ inline int visw(int W) { return (((W + 31) >> 5) + 3) & ~3; }
 
-// Scratch of one walker's batch: the ratio table (9 rows of 80 bytes), 16 step pairs, the 16
-// entries the walk leaves, and the ring of proposals drawn ahead.
+// Scratch of one walker's batch: the ratio table (9 rows of 80 bytes, and 9 of 36 floats), masks and
+// bin changes of the steps, visit counts of the cached bins, the ring of proposals drawn ahead and
+// four control words.
 constexpr int MOVE_TAB_BYTES = 9 * 80;
 constexpr int MOVE_RING = 128;
-constexpr int MOVE_SCRATCH_BYTES = MOVE_TAB_BYTES + (2 * 16 + MOVE_RING) * 16;
-// Largest ln f at which a batch is walked through the ratio table.
-constexpr float TABLE_WALK_LNF = 0x1p-8f;
-// Growth of ln g (visits x ln f) after which the ratio table is taken anew.
-constexpr float TABLE_DRIFT = 0x1p-10f;
-// Cache offsets of the current bin between which the cached bins stay.
-constexpr int CACHE_LO = 8, CACHE_HI = 23;
-// Smallest lattices whose batches are 32 and 16 steps (smaller ones: 8).
+constexpr int MOVE_SCRATCH_BYTES = MOVE_TAB_BYTES + 9 * 36 * 4 + 24 * 16 + 32 * 4 + MOVE_RING * 20 + 16;
+// Largest ln f at which a batch is walked through the ratio table.  Above it the visits of the batch
+// itself leave too many steps undecided (us per launch, Potts L=80 64 x 16 and Ising L=64 32 x 16,
+// table / running walk: 522 / 638 and 440 / 455 at 2^-8, 632 / 639 and 556 / 454 at 2^-7).
+constexpr float TABLE_WALK_LNF = 0x1.8p-8f;
+// Growth of ln g (visits x ln f) after which the ratio table is taken anew: taking it costs about 300
+// cycles, a step left undecided twice that (us per launch at 2^-10 / 2^-6 / 2^-4: Ising L=32 8 x 8
+// at ln f = 2^-12 372 / 341 / 363, Ising L=8 whole run 1099 / 954 / 936).
+constexpr float TABLE_DRIFT = 0x1p-6f;
+// Cache offsets of the current bin between which the cached bins stay (8 .. 23: 1 % slower; a step
+// changes the bin by 4 at most).
+constexpr int CACHE_LO = 6, CACHE_HI = 25;
+// Smallest lattices whose batches are 32 and 16 steps (smaller ones: 8).  Sites soon repeat on a
+// small lattice: a batch ends after about 5 steps on 64 sites, 13 on 256, 24 on 1024.
 constexpr int BATCH32_SITES = 450, BATCH16_SITES = 100;
 
-// Shared memory of one walker in the move kernel: lattice (a 16-bit cell per site, padded to 16
-// sites), int64 ln g shadow over the window (padded to 4 bins; the visit counts are recovered
+// Shared memory of one walker in the move kernel: lattice and stamps (a byte each per site, padded
+// to 16 sites), int64 ln g shadow over the window (padded to 4 bins; the visit counts are recovered
 // from it), the visited-bin bit set, the batch scratch.
 __host__ __device__ inline size_t move_smem_per_walker(int N, int W)
 {
     return 2u * (size_t)((N + 15) & ~15) + (size_t)((W + 3) & ~3) * 8u + (size_t)visw(W) * 4u +
            (size_t)MOVE_SCRATCH_BYTES;
+}
+// Whether a second warp per walker pays: it takes the drawing off the walker's chain, as long as
+// all walkers of the launch are still resident at once (128 registers: 16 warps per SM).
+inline bool draw_ahead_pays(long long walkers, int sms, int walkers_per_cta, size_t smem_per_walker)
+{
+    const long long fit = (long long)(MAX_SMEM_PER_CTA / smem_per_walker);
+    return walkers_per_cta <= 8 && walkers <= sms * (fit < 8 ? fit : 8);
 }
 // The largest lattice and window accepted: 3 bytes per site and 8 per bin within one CTA, which
 // covers move_smem_per_walker for every size it admits.
@@ -103,8 +118,8 @@ __host__ __device__ inline size_t move_smem_per_thread_walker(int N, int W)
 }
 cudaError_t launch_move(const State &s, const MoveCfg &c, cudaStream_t st);
 // Batched instances: states/jobs/tables are device arrays (see the kernels).
-cudaError_t launch_move_batch(const State *states, const int4 *jobs, int njobs, int walkers_per_block,
-                              size_t smem, const MoveCfg &c, cudaStream_t st);
+cudaError_t launch_move_batch(const State *states, const int4 *jobs, int njobs, size_t smem, const MoveCfg &c,
+                              cudaStream_t st);
 cudaError_t launch_check_batch(const State *states, const int2 *tab, int n, const double2 *prm,
                                cudaStream_t st);
 cudaError_t launch_swap_batch(const State *states, const int2 *tab, int n, cudaStream_t st);

@@ -96,3 +96,19 @@ def test_prep_bit_exact(model, L, width, budget):
     for f in gs:
         assert np.array_equal(gs[f], os_[f]), f
     g.close()
+
+
+# more walkers than a second warp each fits the chip: one warp draws and walks
+@pytest.mark.parametrize("model,L,h,m", [(0, 6, 2, 700), (10, 22, 4, 310)])
+def test_many_walkers_bit_exact(model, L, h, m):
+    g, o = _pair(model, L, h, m, seed=I.seed_for(9, L), interval=150)
+    g.init()
+    assert o.init() == 0
+    g.run(max_rounds=2)
+    o.run(2)
+    g.set_state("lnf", np.full(h, 2.0 ** -12))
+    o.put_window(lnf=np.full(h, 2.0 ** -12))
+    g.run(max_rounds=1)
+    o.run(1)
+    _same(g.state(), o.state(), FIELDS)
+    g.close()
