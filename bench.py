@@ -339,7 +339,7 @@ def run_gpu_batch(args, wl, rank, world):
         "e2e": {"value": attempts / e2e_s, "unit": UNIT, "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": d2h // max(args.steps, 1),
                 "call": f"rewl_batch_run({RPS} rounds) + rewl_get_state(lng_mean) of each instance"},
-        "gpu_launches": 4 * RPS * args.steps, "clocks": clk.summary(),
+        "gpu_launches": 2 * RPS * args.steps, "clocks": clk.summary(),
     }
 
 
@@ -788,7 +788,7 @@ def run_gpu(args, wl, rank, world):
         "e2e": {"value": attempts / e2e_s, "unit": UNIT, "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": lng_bytes + 48,
                 "call": f"rewl_run({RPS} rounds) + rewl_get_state(lng_mean) per step"},
-        "gpu_launches": 4 * RPS * args.steps,
+        "gpu_launches": 2 * RPS * args.steps,
         "clocks": clocks,
         "exact_fraction": st["exact_decisions"] / max(st["attempts"], 1),
     }
@@ -849,7 +849,7 @@ def run_gpu_sharded(args, wl, rank, world):
         "config": dict(workload_config(args, wl, 1), parallelism=f"windows{world}"),
         "step_work": {"rounds": RPS, "attempts": per_round * RPS},
         "roofline": _roofline(h.nw * wl["interval"], move_ms, move_launches, sms, step_ms, args.workload),
-        "gpu_launches": (4 + 4 * nb) * RPS * args.steps,
+        "gpu_launches": (2 + 4 * nb) * RPS * args.steps,
         "shards": S.split_windows(wl["windows"], world),
         "transport": dist.get_backend(), "clocks": clk.summary(),
     }

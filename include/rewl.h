@@ -367,7 +367,7 @@ int rewl_join_em(const double *S, int h, int W, int B, int N1, const int *lo_hi,
  * Batched instances.  Many independent REWL simulations (any mix of models, L, window
  * counts, walkers per window; each with its own seed and instance id) advanced together,
  * round by round: one move-kernel launch whose CTAs each serve up to `walkers_per_block`
- * walkers of one instance, then batched flatness/advance, exchange and round-end kernels,
+ * walkers of one instance, then one kernel for flatness/advance, exchange and round end,
  * rounds captured in CUDA graphs.  Every instance evolves bit for bit as it would alone with
  * rewl_create/rewl_run (same parameters, seed, instance id and interval).
  */

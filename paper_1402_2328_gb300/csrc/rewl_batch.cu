@@ -1,7 +1,8 @@
 // rewl_batch.cu -- many independent REWL instances (uneven lattice size, model, window count,
 // walkers per window) advanced together: one move-kernel launch over a job grid (each CTA
-// serves up to `walkers_per_block` walkers of one instance), then batched flatness/advance,
-// exchange and round-end kernels driven by index tables; rounds are captured in CUDA graphs.
+// serves up to `walkers_per_block` walkers of one instance), then one kernel for
+// flatness/advance, exchange and the end of the round, driven by an index table; rounds are
+// captured in CUDA graphs.
 // Every instance evolves exactly as it would alone (its own seed, instance id and state).
 #include <algorithm>
 #include <chrono>
@@ -29,9 +30,9 @@ struct rewl_batch_s {
     // device tables
     State *d_states = nullptr;
     int4 *d_jobs = nullptr;
-    int2 *d_chk = nullptr, *d_swp = nullptr;
+    int2 *d_chk = nullptr;
     double2 *d_prm = nullptr;
-    int njobs = 0, nchk = 0, nswp = 0, block_walkers = 1, wpb_used = 4;
+    int njobs = 0, nchk = 0, block_walkers = 1, wpb_used = 4;
     size_t smem = 0;
     std::vector<DevStatus> hst;
     DevStatus *h_status = nullptr; // pinned, one per instance
@@ -61,11 +62,10 @@ static void free_tables(rewl_batch_t b)
     cudaFree(b->d_states);
     cudaFree(b->d_jobs);
     cudaFree(b->d_chk);
-    cudaFree(b->d_swp);
     cudaFree(b->d_prm);
     b->d_states = nullptr;
     b->d_jobs = nullptr;
-    b->d_chk = b->d_swp = nullptr;
+    b->d_chk = nullptr;
     b->d_prm = nullptr;
 }
 
@@ -173,10 +173,7 @@ static cudaError_t enqueue_batch_round(rewl_batch_t b)
         e = cudaEventRecord(ev.second, b->stream);
         b->ev_used.push_back(ev);
     }
-    const int n = (int)b->inst.size();
-    if (e == cudaSuccess) e = launch_check_batch(b->d_states, b->d_chk, b->nchk, b->d_prm, b->stream);
-    if (e == cudaSuccess) e = launch_swap_batch(b->d_states, b->d_swp, b->nswp, b->stream);
-    if (e == cudaSuccess) e = launch_round_end_batch(b->d_states, n, b->stream);
+    if (e == cudaSuccess) e = launch_round_tail_batch(b->d_states, b->d_chk, b->nchk, b->d_prm, b->stream);
     return e;
 }
 
@@ -300,28 +297,23 @@ int rewl_batch_init(rewl_batch_t b)
     }
     free_tables(b);
     std::vector<State> states(n);
-    std::vector<int2> chk, swp;
+    std::vector<int2> chk;
     std::vector<double2> prm(n);
     for (int i = 0; i < n; ++i) {
         const rewl_t r = b->inst[i];
         states[i] = r->st;
         prm[i] = make_double2(r->flatness, r->lnf_final);
         for (int w = 0; w < r->h; ++w) chk.push_back(make_int2(i, w));
-        for (int p = 0; p < (r->h + 1) / 2 && r->h > 1; ++p) swp.push_back(make_int2(i, p));
     }
     cudaError_t e = cudaMalloc(&b->d_states, n * sizeof(State));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_prm, n * sizeof(double2));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_chk, std::max<size_t>(1, chk.size()) * sizeof(int2));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_swp, std::max<size_t>(1, swp.size()) * sizeof(int2));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_states, states.data(), n * sizeof(State), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_prm, prm.data(), n * sizeof(double2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !chk.empty())
         e = cudaMemcpy(b->d_chk, chk.data(), chk.size() * sizeof(int2), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !swp.empty())
-        e = cudaMemcpy(b->d_swp, swp.data(), swp.size() * sizeof(int2), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return b->cuda_fail(e, "rewl_batch_init tables");
     b->nchk = (int)chk.size();
-    b->nswp = (int)swp.size();
     const int rc = build_jobs(b, b->wpb > 0 ? b->wpb : auto_wpb(b), b->thread_sites);
     if (rc != REWL_OK) return rc;
     b->inited = true;

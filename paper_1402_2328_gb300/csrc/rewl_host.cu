@@ -107,7 +107,7 @@ static void release(rewl_t r)
     State &s = r->st;
     void *ptrs[] = {s.spins, s.cfg, s.k, s.lng, s.H, s.step, s.acc, s.pstep, s.restarts, s.flat,
                     r->d_lohi, s.lnf, s.iter, s.finished, s.mask, s.swap_att, s.swap_acc,
-                    s.it1_round, s.mode, s.frag, s.hem, s.status, r->d_mean, r->d_out, r->d_joins,
+                    s.it1_round, s.mode, s.frag, s.hem, s.status, s.sync, r->d_mean, r->d_out, r->d_joins,
                     r->d_ok};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -167,6 +167,7 @@ static int allocate(rewl_t r)
     s.mode = dmalloc<uint8_t>(h, e);
     s.frag = dmalloc<double>(nw * W, e);
     s.status = dmalloc<DevStatus>(1, e);
+    s.sync = dmalloc<unsigned>((h + 1) / 2 + 1, e);
     r->d_mean = dmalloc<double>(h * W, e);
     r->d_out = dmalloc<double>((size_t)r->B + 1, e);
     r->d_joins = dmalloc<int>(h, e);
@@ -501,9 +502,7 @@ cudaError_t rewl_enqueue_round(rewl_t r)
         r->ev_used.push_back(ev);
     }
     if (e == cudaSuccess && r->st.hem) e = launch_measure_em(r->st, r->stream);
-    if (e == cudaSuccess) e = launch_check(r->st, r->flatness, r->lnf_final, r->stream);
-    if (e == cudaSuccess) e = launch_swap(r->st, r->stream);
-    if (e == cudaSuccess) e = launch_round_end(r->st, r->stream);
+    if (e == cudaSuccess) e = launch_round_tail(r->st, r->flatness, r->lnf_final, r->stream);
     return e;
 }
 

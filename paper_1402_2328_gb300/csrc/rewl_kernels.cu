@@ -4,9 +4,9 @@
 //                 memory; up to 32 proposals are evaluated in parallel, then resolved in
 //                 order (the batch ends before a proposal whose neighbourhood an earlier accepted
 //                 flip touched), so the result equals the one-move-at-a-time walk exactly.
-//   k_check       per-walker flatness (warp-shuffle min / sum over visited bins) and window
-//                 advance: average ln g over the m walkers, H = 0, ln f /= 2 (Sec. 2).
-//   k_swap        replica exchange between windows (w, w+1), Eq. (1).
+//   k_round_tail  per-walker flatness (warp-shuffle min / sum over visited bins) and window
+//                 advance: average ln g over the m walkers, H = 0, ln f /= 2 (Sec. 2); replica
+//                 exchange between windows (w, w+1), Eq. (1); end of the round.
 //   k_init_prep   seeded lattices and the walk into the window.
 //   k_stitch      joining of Sec. 3, Eq. (2).
 #include <cfloat>
@@ -247,8 +247,14 @@ cudaError_t launch_init_prep(const State &s, long long prep_budget, cudaStream_t
 }
 
 // ---------------------------------------------------------------------------------------
-// Flatness + window advance (Sec. 2).  One CTA per window.
+// The rest of a round after the moves, in one launch: flatness and window advance (one CTA per
+// window), replica exchange (by whichever CTA of a window pair comes second), end of the round (by
+// the last CTA).  No CTA waits for another: each passes an arrival counter and goes on or leaves.
+// As three launches (13 + 8 + 3 us and the gaps between them) this took 19 us of a round of Ising
+// L=64 32 x 16, as one 11 us; what is left is launch latency and chains of dependent L2 loads.
 // ---------------------------------------------------------------------------------------
+
+// Flatness + window advance (Sec. 2).
 __device__ __forceinline__ void check_window(const State &s, const int w, const double flatness,
                                              const double lnf_final)
 {
@@ -345,40 +351,8 @@ __device__ __forceinline__ void check_window(const State &s, const int w, const 
     }
 }
 
-__global__ void k_check(State s, double flatness, double lnf_final)
-{
-    check_window(s, blockIdx.x, flatness, lnf_final);
-}
-
-// tab[b] = (instance, window); prm[instance] = (flatness, ln f_final)
-__global__ void k_check_batch(const State *__restrict__ states, const int2 *__restrict__ tab,
-                              const double2 *__restrict__ prm)
-{
-    const int2 t = tab[blockIdx.x];
-    const State s = states[t.x];
-    const double2 p = prm[t.x];
-    check_window(s, t.y, p.x, p.y);
-}
-
-cudaError_t launch_check_batch(const State *states, const int2 *tab, int n, const double2 *prm,
-                               cudaStream_t st)
-{
-    if (n <= 0) return cudaSuccess;
-    k_check_batch<<<n, 512, 0, st>>>(states, tab, prm);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_check(const State &s, double flatness, double lnf_final, cudaStream_t st)
-{
-    k_check<<<s.h, 512, 0, st>>>(s, flatness, lnf_final);
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------------------
-// Replica exchange (Eq. 1) between windows (w, w+1), w = round mod 2.  One warp per pair;
-// lane 0 draws the partner permutation and the decisions (m is small), the swap itself
-// exchanges configuration indices and bins.
-// ---------------------------------------------------------------------------------------
+// Replica exchange (Eq. 1) between windows (w, w+1), w = round mod 2.  One warp per pair; the
+// swap itself exchanges configuration indices and bins.
 // Partner permutation of the exchange of pair (gw, gw+1) in round rd (global window index gw):
 // Fisher-Yates from Philox draws (i, rd, gw, swap tag), i = m-1 .. 1.  One warp; perm in shared
 // memory, valid after the call for every lane.
@@ -414,16 +388,12 @@ __device__ __forceinline__ bool exchange_accept(const State &s, int gw, long lon
     return lnu64(r.x) < lnP;
 }
 
-__device__ __forceinline__ void swap_pair(const State &s, const int pair)
+// The exchange of windows (w, w+1) in round rd, by one warp: the permutation's random draws and the
+// m decisions are lane-parallel (each decision touches its own two walker slots); only the
+// Fisher-Yates swaps themselves run in order.  Other CTAs of the launch wrote some of what is read
+// here, so loads go past the L1.
+__device__ __forceinline__ void swap_windows(const State &s, const int w, const long long rd)
 {
-    // one warp per window pair: the permutation's random draws and the m exchange decisions
-    // are lane-parallel (each decision touches its own two walker slots); only the
-    // Fisher-Yates swaps themselves run in order.  Pairs (w, w+1) with the global window
-    // index w0 + w of the parity of the round.
-    if (s.status->done) return;
-    const long long rd = s.status->round;
-    const int w = 2 * pair + (int)((rd + s.w0) & 1);
-    if (w + 1 >= s.h) return;
     const int lane = threadIdx.x & 31;
     const int m = s.m, W = s.W;
     __shared__ int perm[MAX_M];
@@ -433,11 +403,11 @@ __device__ __forceinline__ void swap_pair(const State &s, const int pair)
     unsigned acc = 0;
     for (int i = lane; i < m; i += 32) {
         const int a = w * m + i, b = (w + 1) * m + perm[i];
-        const int kx = s.k[a], ky = s.k[b];
+        const int kx = __ldcg(s.k + a), ky = __ldcg(s.k + b);
         if (kx < loB || kx > hiB || ky < loA || ky > hiA) continue;
         const double *ga = s.lng + (size_t)a * W, *gb = s.lng + (size_t)b * W;
-        const double lnP = __dadd_rn(__dsub_rn(ga[kx - loA], ga[ky - loA]),
-                                     __dsub_rn(gb[ky - loB], gb[kx - loB]));
+        const double lnP = __dadd_rn(__dsub_rn(__ldcg(ga + (kx - loA)), __ldcg(ga + (ky - loA))),
+                                     __dsub_rn(__ldcg(gb + (ky - loB)), __ldcg(gb + (kx - loB))));
         if (exchange_accept(s, s.w0 + w, rd, i, lnP)) {
             const int t = s.cfg[a];
             s.cfg[a] = s.cfg[b];
@@ -454,27 +424,76 @@ __device__ __forceinline__ void swap_pair(const State &s, const int pair)
     }
 }
 
-__global__ void k_swap(State s) { swap_pair(s, blockIdx.x); }
+// Arrival of this CTA at a counter, after everything its threads wrote: the number of CTAs that came
+// before it.  What those wrote can be read after the call.
+__device__ __forceinline__ unsigned arrive(unsigned *counter)
+{
+    __shared__ unsigned before;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        before = atomicAdd(counter, 1u);
+        __threadfence();
+    }
+    __syncthreads();
+    return before;
+}
 
-// tab[b] = (instance, pair index)
-__global__ void k_swap_batch(const State *__restrict__ states, const int2 *__restrict__ tab)
+// Window w's part of the end of a round.  s.sync: one counter per pair of the round, then one for
+// the windows; all zero between launches.
+__device__ __forceinline__ void round_tail(const State &s, const int w, const double flatness, const double lnf_final)
+{
+    if (s.status->done) return;
+    const long long rd = s.status->round;
+    check_window(s, w, flatness, lnf_final);
+    // pairs (a, a+1) with the global window index w0 + a of the parity of the round
+    const int a = ((w + s.w0 - rd) & 1) == 0 ? w : w - 1;
+    if (a >= 0 && a + 1 < s.h) {
+        unsigned *counter = s.sync + (a >> 1);
+        if (arrive(counter) == 1u) {
+            if (threadIdx.x < 32) swap_windows(s, a, rd);
+            if (threadIdx.x == 0) *counter = 0u;
+        }
+    }
+    unsigned *counter = s.sync + (s.h + 1) / 2;
+    if (arrive(counter) != (unsigned)s.h - 1u) return;
+    int open = s.production;
+    for (int i = threadIdx.x; i < s.h; i += blockDim.x) open |= !__ldcg(s.finished + i);
+    const bool all = !__syncthreads_or(open);
+    if (threadIdx.x == 0) {
+        *counter = 0u;
+        s.status->round = rd + 1;
+        if (all) s.status->done = 1;
+    }
+}
+
+__global__ void __launch_bounds__(512) k_round_tail(State s, double flatness, double lnf_final)
+{
+    round_tail(s, blockIdx.x, flatness, lnf_final);
+}
+
+// tab[b] = (instance, window); prm[instance] = (flatness, ln f_final)
+__global__ void __launch_bounds__(512) k_round_tail_batch(const State *__restrict__ states,
+                                                          const int2 *__restrict__ tab,
+                                                          const double2 *__restrict__ prm)
 {
     const int2 t = tab[blockIdx.x];
     const State s = states[t.x];
-    swap_pair(s, t.y);
+    const double2 p = prm[t.x];
+    round_tail(s, t.y, p.x, p.y);
 }
 
-cudaError_t launch_swap_batch(const State *states, const int2 *tab, int n, cudaStream_t st)
+cudaError_t launch_round_tail_batch(const State *states, const int2 *tab, int n, const double2 *prm,
+                                    cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    k_swap_batch<<<n, 32, 0, st>>>(states, tab);
+    k_round_tail_batch<<<n, 512, 0, st>>>(states, tab, prm);
     return cudaGetLastError();
 }
 
-cudaError_t launch_swap(const State &s, cudaStream_t st)
+cudaError_t launch_round_tail(const State &s, double flatness, double lnf_final, cudaStream_t st)
 {
-    if (s.h < 2) return cudaSuccess;
-    k_swap<<<(s.h + 1) / 2, 32, 0, st>>>(s);
+    k_round_tail<<<s.h, 512, 0, st>>>(s, flatness, lnf_final);
     return cudaGetLastError();
 }
 
@@ -614,36 +633,6 @@ cudaError_t launch_bnd_import(const State &s, int side, const int *pbins, const 
                               const int8_t *plat, cudaStream_t st)
 {
     k_bnd_import<<<1, 32, 0, st>>>(s, side, pbins, acc, plat);
-    return cudaGetLastError();
-}
-
-__device__ __forceinline__ void round_end(const State &s)
-{
-    if (s.status->done) return;
-    s.status->round += 1;
-    int all = !s.production;
-    for (int w = 0; w < s.h; ++w) all &= s.finished[w];
-    if (all) s.status->done = 1;
-}
-
-__global__ void k_round_end(State s) { round_end(s); }
-
-__global__ void k_round_end_batch(const State *__restrict__ states, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) round_end(states[i]);
-}
-
-cudaError_t launch_round_end_batch(const State *states, int n, cudaStream_t st)
-{
-    if (n <= 0) return cudaSuccess;
-    k_round_end_batch<<<(n + 63) / 64, 64, 0, st>>>(states, n);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_round_end(const State &s, cudaStream_t st)
-{
-    k_round_end<<<1, 1, 0, st>>>(s);
     return cudaGetLastError();
 }
 

@@ -46,6 +46,7 @@ struct State {
     uint32_t *hem;            // [h][W][N+1] (bin, up spins) counts, nullptr: not measured
     int production;           // rounds continue after every window finished
     DevStatus *status;
+    unsigned *sync;           // [(h+1)/2 + 1] arrival counters of k_round_tail, zero between launches
     uint32_t key0, key1, inst;
     int w0, slot0;            // window-sharded run: global index of window 0 / walker slot 0
 };
@@ -120,14 +121,10 @@ cudaError_t launch_move(const State &s, const MoveCfg &c, cudaStream_t st);
 // Batched instances: states/jobs/tables are device arrays (see the kernels).
 cudaError_t launch_move_batch(const State *states, const int4 *jobs, int njobs, size_t smem, const MoveCfg &c,
                               cudaStream_t st);
-cudaError_t launch_check_batch(const State *states, const int2 *tab, int n, const double2 *prm,
-                               cudaStream_t st);
-cudaError_t launch_swap_batch(const State *states, const int2 *tab, int n, cudaStream_t st);
-cudaError_t launch_round_end_batch(const State *states, int n, cudaStream_t st);
+cudaError_t launch_round_tail_batch(const State *states, const int2 *tab, int n, const double2 *prm,
+                                    cudaStream_t st);
 cudaError_t launch_init_prep(const State &s, long long prep_budget, cudaStream_t st);
-cudaError_t launch_check(const State &s, double flatness, double lnf_final, cudaStream_t st);
-cudaError_t launch_swap(const State &s, cudaStream_t st);
-cudaError_t launch_round_end(const State &s, cudaStream_t st);
+cudaError_t launch_round_tail(const State &s, double flatness, double lnf_final, cudaStream_t st);
 cudaError_t launch_set_done(const State &s, cudaStream_t st);
 // joint density of states g(E, M) (rewl_em.cu)
 cudaError_t launch_measure_em(const State &s, cudaStream_t st);
