@@ -34,7 +34,9 @@ struct rewl_s {
     rewl::State st{};
     int *d_lohi = nullptr;
     double *d_mean = nullptr, *d_out = nullptr;
+    double *d_at = nullptr;
     int *d_joins = nullptr, *d_ok = nullptr;
+    void *d_jack = nullptr; // workspace of rewl_jackknife, made by its first call
     rewl::DevStatus *h_status = nullptr; // pinned
     // graphs
     cudaGraphExec_t graph = nullptr;

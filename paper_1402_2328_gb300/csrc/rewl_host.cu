@@ -108,7 +108,7 @@ static void release(rewl_t r)
     void *ptrs[] = {s.spins, s.cfg, s.k, s.lng, s.H, s.step, s.acc, s.pstep, s.restarts, s.flat,
                     r->d_lohi, s.lnf, s.iter, s.finished, s.mask, s.swap_att, s.swap_acc,
                     s.it1_round, s.mode, s.frag, s.hem, s.status, s.sync, r->d_mean, r->d_out, r->d_joins,
-                    r->d_ok};
+                    r->d_ok, r->d_at, r->d_jack};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (r->h_status) cudaFreeHost(r->h_status);
@@ -117,6 +117,8 @@ static void release(rewl_t r)
     r->d_lohi = nullptr;
     r->d_mean = r->d_out = nullptr;
     r->d_joins = r->d_ok = nullptr;
+    r->d_at = nullptr;
+    r->d_jack = nullptr;
     r->allocated = false;
 }
 
@@ -171,6 +173,7 @@ static int allocate(rewl_t r)
     r->d_mean = dmalloc<double>(h * W, e);
     r->d_out = dmalloc<double>((size_t)r->B + 1, e);
     r->d_joins = dmalloc<int>(h, e);
+    r->d_at = dmalloc<double>(2 * h, e);
     r->d_ok = dmalloc<int>(1, e);
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&r->h_status, sizeof(DevStatus), cudaHostAllocDefault);
     if (e != cudaSuccess) {
@@ -655,22 +658,26 @@ int rewl_jackknife(rewl_t r, double *err, int cap, int norm)
     const double de = r->model == 0 ? 4.0 : 1.0;
     const int step = (r->model != 0 && r->q == 2) ? 2 : 1;
     const double target = norm == 0 ? (double)r->N * std::log((double)r->q) : std::log((double)r->q);
-    double *theta = nullptr, *d_err = nullptr;
-    cudaError_t e = cudaMalloc(&theta, (size_t)r->m * (r->B + 1) * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&d_err, (size_t)(r->B + 1) * 8);
-    std::vector<int> oks((size_t)r->m, 0);
-    for (int j = 0; j < r->m && e == cudaSuccess; ++j) {
-        e = launch_loo_mean(r->st, j, r->d_mean, r->stream);
-        if (e == cudaSuccess)
-            e = launch_stitch(r->st, r->d_mean, de, step, norm, target, theta + (size_t)j * (r->B + 1),
-                              r->d_joins, r->d_ok, r->B, r->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&oks[j], r->d_ok, sizeof(int), cudaMemcpyDeviceToHost, r->stream);
+    // workspace: the m resamples' values at their joins (16-byte aligned), window means and joined ln g, the
+    // error, joins and flags
+    const size_t m = (size_t)r->m, h = (size_t)r->h, W = (size_t)r->W, nb = (size_t)r->B + 1;
+    const size_t doubles = 2 * m * h + m * h * W + m * nb + nb, ints = m * h + m;
+    cudaError_t e = cudaSuccess;
+    if (!r->d_jack) e = cudaMalloc(&r->d_jack, doubles * 8 + ints * 4);
+    if (e != cudaSuccess) {
+        r->d_jack = nullptr;
+        return r->cuda_fail(e, "rewl_jackknife");
     }
+    double *at = (double *)r->d_jack, *means = at + 2 * m * h, *theta = means + m * h * W, *d_err = theta + m * nb;
+    int *joins = (int *)(d_err + nb), *d_oks = joins + m * h;
+    std::vector<int> oks(m, 0);
+    e = launch_loo_mean(r->st, means, r->stream);
+    if (e == cudaSuccess)
+        e = launch_stitch(r->st, r->m, means, de, step, norm, target, theta, joins, at, d_oks, r->B, r->stream);
     if (e == cudaSuccess) e = launch_jack(theta, r->m, r->B, d_err, r->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(err, d_err, (size_t)(r->B + 1) * 8, cudaMemcpyDeviceToHost, r->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(oks.data(), d_oks, m * sizeof(int), cudaMemcpyDeviceToHost, r->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(err, d_err, nb * 8, cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
-    cudaFree(theta);
-    cudaFree(d_err);
     if (e != cudaSuccess) return r->cuda_fail(e, "rewl_jackknife");
     for (int ok : oks)
         if (!ok) return r->fail(REWL_ERR_NOT_CONVERGED, "rewl_jackknife: a resample cannot be joined");
@@ -893,8 +900,8 @@ int rewl_stitch(rewl_t r, double *out, int cap, int norm, int *joins)
     const double target = norm == 0 ? (double)r->N * std::log((double)r->q) : std::log((double)r->q);
     cudaError_t e = launch_window_mean(r->st, r->d_mean, r->stream);
     if (e == cudaSuccess)
-        e = launch_stitch(r->st, r->d_mean, de, step, norm, target, r->d_out, r->d_joins, r->d_ok,
-                          r->B, r->stream);
+        e = launch_stitch(r->st, 1, r->d_mean, de, step, norm, target, r->d_out, r->d_joins, r->d_at,
+                          r->d_ok, r->B, r->stream);
     int ok = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, r->d_out, (size_t)(r->B + 1) * 8, cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&ok, r->d_ok, sizeof(int), cudaMemcpyDeviceToHost, r->stream);

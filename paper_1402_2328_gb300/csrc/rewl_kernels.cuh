@@ -129,9 +129,10 @@ cudaError_t launch_set_done(const State &s, cudaStream_t st);
 // joint density of states g(E, M) (rewl_em.cu)
 cudaError_t launch_measure_em(const State &s, cudaStream_t st);
 cudaError_t launch_window_mean(const State &s, double *out /*[h][W]*/, cudaStream_t st);
-cudaError_t launch_stitch(const State &s, const double *mean, double de, int step, int norm,
-                          double target, double *out /*B+1*/, int *joins /*h-1*/,
-                          int *ok /*1*/, int B, cudaStream_t st);
+// n joins at once: of the window means at mean + r h W, r = 0 .. n-1
+cudaError_t launch_stitch(const State &s, int n, const double *mean, double de, int step, int norm,
+                          double target, double *out /*[n][B+1]*/, int *joins /*[n][h]*/, double *at /*[n][h][2]*/,
+                          int *ok /*[n]*/, int B, cudaStream_t st);
 
 // window-sharded runs: the exchange of the pair across a shard boundary (Eq. 1), in four steps
 // (side 1: this shard holds the pair's lower window, its last; side 0: the upper, its first)
@@ -142,7 +143,7 @@ cudaError_t launch_bnd_decide(const State &s, int side, const double *half, cons
                               uint8_t *acc, int8_t *lat_out, cudaStream_t st);
 cudaError_t launch_bnd_import(const State &s, int side, const int *pbins, const uint8_t *acc,
                               const int8_t *plat, cudaStream_t st);
-cudaError_t launch_loo_mean(const State &s, int j, double *out /*[h][W]*/, cudaStream_t st);
+cudaError_t launch_loo_mean(const State &s, double *out /*[m][h][W]*/, cudaStream_t st);
 cudaError_t launch_jack(const double *theta /*[m][B+1]*/, int m, int B, double *err, cudaStream_t st);
 cudaError_t launch_thermo(const double *lng, int model, int L, const double *T, int nT, double *U,
                           double *C, cudaStream_t st);
