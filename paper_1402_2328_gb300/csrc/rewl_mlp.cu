@@ -77,7 +77,7 @@ __global__ void k_mlp_forward(const float *__restrict__ P, const float *__restri
 // weight gradient; 256 threads with 4 x 4 outputs each, operands in 16-byte loads from rows of ROW
 // floats, which meets every bank once) and by the latency of the phases between them.  With 64
 // samples a CTA the documented 9716 samples give 152 CTAs, one per SM.  One step (gradient, reduction,
-// Adam) on 9716 samples: 105 us with one thread per sample and 128 samples a CTA, @MLP@ us.
+// Adam) on 9716 samples: 105 us with one thread per sample and 128 samples a CTA, 22 us.
 constexpr int SUB = 64;
 constexpr int ROW = HID + 4;
 constexpr int GT = 256; // threads of the gradient kernel
@@ -90,7 +90,7 @@ struct GradMem {
     float D2[SUB * ROW];  // h2[s][i], then dz2[s][i]
     float g[(NPARAM + 3) & ~3]; // this CTA's gradient
     float W1[HID * 3], b1[HID], b2[HID], W3[HID];
-    float x[SUB * 3], dy[SUB], r2[SUB];
+    float x[SUB * 3], target[SUB], dy[SUB], r2[SUB];
 };
 
 // acc[a][b] += sum_k A[ts + 16 a][k] Bm[ti + 16 b][k] over k < 64
@@ -124,20 +124,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GT)
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int t = threadIdx.x, ti = t & 15, ts = t >> 4;
     const int base = blockIdx.x * SUB, tile = blockIdx.x >> 1;
-    for (int e = t; e < HID * HID; e += GT) {
-        const float w = P[OFF_W2 + e];
-        M.W2[(e / HID) * ROW + e % HID] = w;
-        M.W2T[(e % HID) * ROW + e / HID] = w;
-    }
+    float w2[HID * HID / GT]; // all loads in flight at once
+#pragma unroll
+    for (int k = 0; k < HID * HID / GT; ++k) w2[k] = P[OFF_W2 + t + k * GT];
     if (t < HID * 3) M.W1[t] = P[OFF_W1 + t];
     if (t < HID) {
         M.b1[t] = P[OFF_B1 + t];
         M.b2[t] = P[OFF_B2 + t];
         M.W3[t] = P[OFF_W3 + t];
     }
+    if (t < SUB) M.target[t] = base + t < n ? T[base + t] : 0.f;
     if (t < SUB * 3) M.x[t] = base + t / 3 < n ? X[3 * (size_t)base + t] : 0.f;
     const float b3 = P[OFF_B3];
+#pragma unroll
+    for (int k = 0; k < HID * HID / GT; ++k) {
+        const int e = t + k * GT;
+        M.W2[(e / HID) * ROW + e % HID] = w2[k];
+        M.W2T[(e % HID) * ROW + e / HID] = w2[k];
+    }
     __syncthreads();
+#pragma unroll 4
     for (int e = t; e < SUB * HID; e += GT) { // layer 1
         const int q = e / HID, j = e % HID;
         const float z = M.b1[j] + M.W1[3 * j] * M.x[3 * q] + M.W1[3 * j + 1] * M.x[3 * q + 1] + M.W1[3 * j + 2] * M.x[3 * q + 2];
@@ -164,8 +170,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GT)
         for (int o = 8; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
         y += b3;
         if (ti == 0) {
-            const bool live = base + q < n;
-            const float r = live ? y - T[base + q] : 0.f;
+            const float r = base + q < n ? y - M.target[q] : 0.f;
             M.dy[q] = 2.0f * r / (float)n;
             M.r2[q] = r * r;
         }
@@ -234,8 +239,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GT)
         }
 #pragma unroll
         for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) M.g[OFF_W2 + (4 * ts + a) * HID + 4 * ti + b] = acc[a][b];
+            *reinterpret_cast<float4 *>(M.g + OFF_W2 + (4 * ts + a) * HID + 4 * ti) =
+                make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
     }
     {
         const float g = over_samples([&](int q) { return M.D2[q * ROW + u]; });
@@ -251,9 +256,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GT)
     const unsigned rank = cluster.block_rank();
     const GradMem &O = *cluster.map_shared_rank(&M, rank ^ 1u);
     float *out = partial + (size_t)tile * NPARAM;
-    for (int p = t + (rank ? NPARAM / 2 : 0); p < (rank ? NPARAM : NPARAM / 2); p += GT) {
-        const float mine = M.g[p], other = O.g[p];
-        out[p] = rank ? other + mine : mine + other;
+    float other[NPARAM / 2 / GT + 1]; // all loads in flight at once
+#pragma unroll
+    for (int k = 0; k < NPARAM / 2 / GT + 1; ++k) {
+        const int p = t + k * GT + (rank ? NPARAM / 2 : 0);
+        other[k] = p < (rank ? NPARAM : NPARAM / 2) ? O.g[p] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < NPARAM / 2 / GT + 1; ++k) {
+        const int p = t + k * GT + (rank ? NPARAM / 2 : 0);
+        if (p < (rank ? NPARAM : NPARAM / 2)) out[p] = rank ? other[k] + M.g[p] : M.g[p] + other[k];
     }
     if (rank == 0 && t == 0) loss_partial[tile] = M.r2[0] + O.r2[0];
     cluster.sync(); // the other CTA has read this one's sums
@@ -285,7 +297,7 @@ __global__ void __launch_bounds__(RED_P *RED_S)
     const int i = threadIdx.x % RED_P, q = threadIdx.x / RED_P, p = blockIdx.x * RED_P + i;
     float g = 0.f;
     if (p < NPARAM)
-#pragma unroll 4
+#pragma unroll 10
         for (int k = q; k < ntiles; k += RED_S) g += partial[(size_t)k * NPARAM + p];
     sums[q][i] = g;
     __syncthreads();
