@@ -66,9 +66,9 @@ __device__ __forceinline__ int propose_dk(const int8_t *sp, const Lattice &lat, 
 //      is too close as well, on the shadow or in float64.
 //      Large ln f, where each visit turns later decisions: the path is walked with running
 //      float32 values through shuffles, every step screened by the same kind of margin;
-//   4. the batch is cut before the first step that has a neighbour changed by an earlier step of
-//      the batch, or shares its site with one, and behind it the side effects (spin flips, visits)
-//      are applied lane-parallel.
+//   4. the batch is cut before the first step whose site or a neighbour of it an earlier step of
+//      the batch changed, and the side effects (spin flips, visits) of the steps before the cut are
+//      applied lane-parallel.
 // A step inside every margin is decided from the float64 values rebuilt exactly (seqadd of
 // the interval-start ln g and the visit counts); at the end of the launch the float64 ln g of
 // every bin is rebuilt the same way, so the state equals that of the sequential walk bit for bit.
@@ -159,7 +159,7 @@ constexpr unsigned NO_CLAIM = 0xffu; // stamp of a site that the last drawn bloc
 
 struct WalkerMem {
     uint8_t *sp;        // [N] lattice
-    uint8_t *stamp;     // [N] lane of the last drawn block that proposes the site last
+    uint8_t *stamp;     // [N] last lane of the block drawn last that proposes the site
     long long *V;       // [W] shadow of ln g
     uint32_t *vis;      // [W bits] bin visited
     unsigned char *tab; // ratio table
@@ -244,38 +244,50 @@ __device__ __forceinline__ void draw_words(const State &s, const MoveCfg &c, int
     }
 }
 
+// The block of 32 steps drawn before: each lane's site, and the lanes whose site a later lane of the block
+// proposes again (their stamps are gone).
+struct Drawn {
+    int site = -1;
+    unsigned hidden = 0u;
+};
+
 // Proposals of steps g .. g+31 (lane j: step g + j) into the ring: site, new-state draw, the four
-// neighbours, ln u, and which earlier steps they meet:
-//   - how many steps ago the site was proposed last (bits 24.. of x; 63: not in the last 31),
-//   - `near`: bit 32 - d set if one of the neighbours was proposed last d steps ago, d <= 31.
-// Only the last proposal of a site counts: a batch ends before a step whose site an earlier step
-// of the batch proposes too, so no step meets two proposals of one neighbour in its batch.
-// `stamp` holds, between calls, the lanes of the block drawn before; psite is that block's site.
+// neighbours, ln u; and into `near` which of the 31 steps before propose the site or one of its
+// neighbours: bit 32 - d for the one d steps ago.
+// `stamp` holds, between calls, for every site the last lane of the block before that proposes it.
 template <bool ISING, bool REPLAY>
 __device__ __forceinline__ void draw_block(const State &s, const MoveCfg &c, const WalkerMem &mem, int slot,
-                                           unsigned long long st0, int g, int &psite, int lane)
+                                           unsigned long long st0, int g, Drawn &before, int lane)
 {
     uint32_t w0, w1, w2;
     draw_words<REPLAY>(s, c, slot, st0, g + lane, w0, w1, w2);
     const int site = (int)mulhi(w0, (uint32_t)s.N);
     const Lattice lat{s.L, s.N, s.magic};
-    int nb[4];
+    int nb[5];
     lat.nbrs(site, nb[0], nb[1], nb[2], nb[3]);
+    nb[4] = site;
     const unsigned pr = ISING ? 0u : mulhi(w1, (uint32_t)(s.q - 1));
     const float lnu = lnu32(w2);
-    // the block before: lane l there is 32 + lane - l steps ago
-    int od = 32 + lane - (int)mem.stamp[site], dist[4]; // NO_CLAIM gives a negative number
+    auto meets = [&](int sl) { return sl == nb[0] || sl == nb[1] || sl == nb[2] || sl == nb[3] || sl == nb[4]; };
+    unsigned near = 0u;
+    // the block before: lane l there is 32 + lane - l steps ago, at most 31 for l > lane (a smaller l
+    // and NO_CLAIM shift the bit out; l = lane sets bit 0, which nothing reads)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) dist[i] = 32 + lane - (int)mem.stamp[nb[i]];
+    for (int i = 0; i < 5; ++i) near |= shl_clamp(1u, (uint32_t)mem.stamp[nb[i]] - (uint32_t)lane);
+    for (unsigned h = before.hidden; h; h &= h - 1) {
+        const int l = __ffs(h) - 1, sl = __shfl_sync(FULL, before.site, l);
+        if (l > lane && meets(sl)) near |= 1u << (l - lane);
+    }
     __syncwarp();
-    if (psite >= 0) mem.stamp[psite] = (uint8_t)NO_CLAIM;
-    psite = site;
+    if (before.site >= 0) mem.stamp[before.site] = (uint8_t)NO_CLAIM;
+    before.site = site;
+    before.hidden = 0u;
     __syncwarp();
     mem.stamp[site] = (uint8_t)lane;
     __syncwarp();
     // two lanes on one site: make the lowest lane's stamp stand
     int own = mem.stamp[site];
-    bool twice = __any_sync(FULL, own != lane);
+    const bool twice = __any_sync(FULL, own != lane);
     if (twice) {
         for (int it = 0; it < 32; ++it) { // each pass lowers some stamp: ends within 32 passes
             const bool again = own > lane;
@@ -286,35 +298,23 @@ __device__ __forceinline__ void draw_block(const State &s, const MoveCfg &c, con
             own = mem.stamp[site];
         }
     }
-    if (own < lane) od = lane - own;
+    // this block: lane l is lane - l steps ago (l >= lane and NO_CLAIM shift the bit out)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int l = mem.stamp[nb[i]];
-        if (l < lane) dist[i] = lane - l;
-    }
-    if (twice) { // later proposals of a site, in order: they are the last ones for the lanes after
+    for (int i = 0; i < 5; ++i) near |= shl_clamp(1u, (uint32_t)(32 - lane) + mem.stamp[nb[i]]);
+    if (twice) { // the later proposals of a site, in order: the last one keeps the stamp
         unsigned late = __ballot_sync(FULL, own < lane);
         while (late) {
-            const int l = __ffs(late) - 1;
+            const int l = __ffs(late) - 1, sl = __shfl_sync(FULL, site, l);
             late &= late - 1;
-            const int sl = __shfl_sync(FULL, site, l);
-            if (lane > l) {
-                if (site == sl) od = lane - l;
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (nb[i] == sl) dist[i] = lane - l;
-            }
+            if (lane > l && meets(sl)) near |= 1u << (32 - lane + l);
             __syncwarp();
             if (lane == l) mem.stamp[site] = (uint8_t)lane;
         }
+        __syncwarp();
+        before.hidden = __ballot_sync(FULL, mem.stamp[site] != lane);
     }
-    unsigned near = 0u;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) // 1 <= dist <= 31, else the shift gives 0 or the bit is not there
-        near |= dist[i] > 0 ? shl_clamp(1u, 32u - (unsigned)dist[i]) : 0u;
-    const unsigned ago = od > 0 && od < 32 ? (unsigned)od : 63u;
     const int e = (g + lane) & (MOVE_RING - 1);
-    mem.ring[e] = make_uint4((unsigned)site | (pr << 16) | (ago << 24), (unsigned)nb[0] | ((unsigned)nb[1] << 16),
+    mem.ring[e] = make_uint4((unsigned)site | (pr << 16), (unsigned)nb[0] | ((unsigned)nb[1] << 16),
                              (unsigned)nb[2] | ((unsigned)nb[3] << 16), __float_as_uint(lnu));
     mem.near[e] = near;
 }
@@ -356,13 +356,13 @@ __device__ __forceinline__ void draw_walker(const State &s, const MoveCfg &c, co
     const unsigned long long st0 = s.step[slot];
     for (int i = lane; i < (pad16(s.N) >> 2); i += 32) reinterpret_cast<uint32_t *>(mem.stamp)[i] = ~0u;
     __syncwarp();
-    int psite = -1;
+    Drawn before;
     for (int g = 0; g < c.T + 64; g += 32) { // the first warp asks for 33 steps beyond the last
         for (int it = 0; g + 32 - load_acquire(mem.ctl + 1) > MOVE_RING; ++it) {
             if (load_acquire(mem.ctl + 2) || it > SPIN_LIMIT) return;
             __nanosleep(50);
         }
-        draw_block<ISING, false>(s, c, mem, slot, st0, g, psite, lane);
+        draw_block<ISING, false>(s, c, mem, slot, st0, g, before, lane);
         __syncwarp();
         if (lane == 0) store_release(mem.ctl, g + 32);
     }
@@ -516,7 +516,8 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
     cache_load(kstart);
     int table_age = table_life + 1; // visits since the table was taken
 
-    int g = 0, psite = -1; // steps drawn (as far as this warp knows)
+    int g = 0; // steps drawn (as far as this warp knows)
+    Drawn before;
     // steps up to `upto` drawn; false if the partner warp does not come
     auto drawn = [&](int upto) -> bool {
         if (AHEAD) {
@@ -524,7 +525,7 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
             return __all_sync(FULL, g >= upto);
         }
         while (g < upto) {
-            draw_block<ISING, REPLAY>(s, c, mem, slot, st0, g, psite, lane);
+            draw_block<ISING, REPLAY>(s, c, mem, slot, st0, g, before, lane);
             g += 32;
             __syncwarp();
         }
@@ -552,11 +553,10 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
         const int site = (int)(pe.x & 0xffffu);
         const unsigned c1 = sp[pe.y & 0xffffu], c2 = sp[pe.y >> 16], c3 = sp[pe.z & 0xffffu], c4 = sp[pe.z >> 16];
         const uint32_t s0 = sp[site];
-        // earlier lanes that propose one of this site's neighbours; settled after the walk: the
-        // batch ends before the first step one of whose neighbours was changed
+        // earlier lanes that propose this site or one of its neighbours; settled after the walk: the
+        // batch ends before the first step one of whose claims was accepted
         const unsigned claims = lane ? pnear >> (32 - lane) : 0u;
-        // an earlier lane proposes the same site: the batch ends before this step
-        const int cut = lane >= n || (pe.x >> 24) <= (unsigned)lane ? -1 : 0;
+        const int cut = lane >= n ? -1 : 0;
         const uint32_t nbytes = __byte_perm(__byte_perm(c1, c2, 0x0040), __byte_perm(c3, c4, 0x0040), 0x5410);
         int snew, dkm;    // dkm = dk + DM
         if (ISING) {
@@ -564,7 +564,7 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
             // dE = 2 s0 sum of neighbours, dk = dE / 4 = 2 - neighbours unequal to s0
             dkm = (int)__dp4a((int)bytes_unequal<true>(nbytes, s0), -1, 4);
         } else {
-            snew = (int)(s0 + 1u + ((pe.x >> 16) & 0xffu));
+            snew = (int)(s0 + 1u + (pe.x >> 16));
             if (snew >= s.q) snew -= s.q;
             dkm = __dp4a((int)bytes_unequal<false>(nbytes, s0), -1,
                          __dp4a((int)bytes_unequal<false>(nbytes, (uint32_t)snew), 0x01010101, DM));
@@ -772,7 +772,7 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
         // ---- side effects of steps 0 .. stop-1
         const bool mine = lane < stop;
         const bool accj = dz || xa != xb; // step j accepted (a move to another bin, or dE = 0)
-        if (mine && accj) sp[site] = (uint8_t)snew; // distinct sites
+        if (mine && accj) sp[site] = (uint8_t)snew; // distinct sites: an accepted claim ends the batch
         if (mine) atomicAdd(&mem.cnt[xa], 1u);
         if (REPLAY && mine) {
             c.acc_out[(size_t)slot * T + t + lane] = accj ? 1 : 0;
