@@ -147,6 +147,74 @@ __device__ __forceinline__ double seqadd(double x, double f, uint32_t c)
     return x;
 }
 
+// The two conversions below are integer arithmetic on the bits: an SM has float64 units for two lanes
+// a cycle, and all its walkers convert their windows at the same time.
+
+// x 2^32 rounded to the nearest integer (ties to even), |x| < 2^30.
+__device__ __forceinline__ long long to_fixed(double x)
+{
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)((bits >> 52) & 0x7ff);
+    const unsigned long long mant = (bits & 0x000fffffffffffffULL) | 0x0010000000000000ULL;
+    const int sh = 52 - (ex - 1023 + 32); // x 2^32 = mant 2^-sh
+    unsigned long long v;
+    if (sh <= 0) {
+        v = mant << (-sh & 63);
+    } else if (sh > 53) { // below 1/2, zero and subnormal numbers too
+        v = 0;
+    } else {
+        const unsigned long long rem = mant & ((1ULL << sh) - 1ULL), half = 1ULL << (sh - 1);
+        v = mant >> sh;
+        v += (rem > half || (rem == half && (v & 1ULL))) ? 1ULL : 0ULL;
+    }
+    return (bits >> 63) ? -(long long)v : (long long)v;
+}
+
+// seqadd for additions that all stay in the binade of x > 0 and do not tie (nearly all of them): false
+// and nothing written for others.  With x = M u (u the spacing of the binade) every addition adds
+// a = f / u rounded to the nearest integer, so the sum is (M + c a) u while that stays below 2^53 u.
+__device__ __forceinline__ bool seqadd_in_binade(double x, double f, uint32_t c, double *out)
+{
+    const unsigned long long xb = (unsigned long long)__double_as_longlong(x), fb = (unsigned long long)__double_as_longlong(f);
+    const int ex = (int)(xb >> 52), ef = (int)(fb >> 52), s = ex - ef; // a sign bit makes ex or ef >= 2048
+    if (ex < 1 || ex > 2046 || ef < 1 || ef > 2046 || s < 0) return false;
+    const unsigned long long M = (xb & 0x000fffffffffffffULL) | 0x0010000000000000ULL;
+    const unsigned long long F = (fb & 0x000fffffffffffffULL) | 0x0010000000000000ULL;
+    unsigned long long a = 0;
+    if (s <= 53) {
+        a = F >> s;
+        if (s > 0) {
+            const unsigned long long rem = F & ((1ULL << s) - 1ULL), half = 1ULL << (s - 1);
+            if (rem == half) return false;
+            a += rem > half ? 1ULL : 0ULL;
+        }
+    }
+    if (__umul64hi(a, (unsigned long long)c) != 0ULL) return false;
+    const unsigned long long add = a * (unsigned long long)c;
+    if (add > 0x001fffffffffffffULL - M) return false;
+    *out = __longlong_as_double((long long)(((unsigned long long)ex << 52) | ((M + add) & 0x000fffffffffffffULL)));
+    return true;
+}
+
+// Exact division of multiples of d > 0 by d, for quotients below 2^32: shift by d's factors of two, then
+// a multiplication by the inverse of the odd part modulo 2^64 (Newton).
+struct ExactDiv {
+    unsigned long long inv;
+    int shift;
+    __device__ __forceinline__ explicit ExactDiv(long long d)
+    {
+        shift = __ffsll(d) - 1;
+        const unsigned long long o = (unsigned long long)d >> shift;
+        inv = o; // right to 3 bits; each step doubles them
+#pragma unroll
+        for (int i = 0; i < 5; ++i) inv *= 2ULL - o * inv;
+    }
+    __device__ __forceinline__ uint32_t operator()(long long x) const
+    {
+        return (uint32_t)(((unsigned long long)x >> shift) * inv);
+    }
+};
+
 // Site -> (x, y) with a multiply-high by ceil(2^32 / L) (exact for site * L < 2^32).
 struct Lattice {
     int L, N;

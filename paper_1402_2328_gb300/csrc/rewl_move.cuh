@@ -116,7 +116,16 @@ __device__ __forceinline__ float warp_maxf(float v)
 // visits of bin b since the launch started: the shadow grew by lnfq per visit
 __device__ __forceinline__ uint32_t visits(const long long *V, const double *glng, int b, long long lnfq)
 {
-    return (uint32_t)((V[b] - __double2ll_rn(__dmul_rn(glng[b], 0x1p32))) / lnfq);
+    return (uint32_t)((V[b] - to_fixed(glng[b])) / lnfq);
+}
+
+// ln g and H of bin b at the end of a launch: v visits since it started
+__device__ __forceinline__ void write_back(double *gl, uint32_t *gH, int b, double lnf, double x, uint32_t v)
+{
+    if (v == 0u) return;
+    if (!seqadd_in_binade(x, lnf, v, &x)) x = seqadd(x, lnf, v);
+    gl[b] = x;
+    gH[b] += v;
 }
 
 // Float64 decision from the exact values (rare): ln g of bins k and k' rebuilt by seqadd from
@@ -406,25 +415,35 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
     if (s.vec_spins) {
         const int4 *src = reinterpret_cast<const int4 *>(gsp);
         int4 *dst = reinterpret_cast<int4 *>(sp);
+#pragma unroll 4
         for (int i = lane; i < (s.N >> 4); i += 32) dst[i] = src[i];
     } else {
+#pragma unroll 4
         for (int i = lane; i < s.N; i += 32) sp[i] = (uint8_t)gsp[i];
     }
     if (!AHEAD)
         for (int i = lane; i < (pad16(s.N) >> 2); i += 32) reinterpret_cast<uint32_t *>(mem.stamp)[i] = ~0u;
-    double mx = 0.0;
-    bool bad_in = false;
+    unsigned long long mxb = 0; // bits of the largest |ln g| (they order like the numbers, NaN above all)
+#pragma unroll 4
     for (int b = lane; b < nb; b += 32) {
         const double x = glng[b];
-        bad_in = bad_in || !(fabs(x) < 0x1p30); // also catches NaN
-        mx = fmax(mx, fabs(x));
-        V[b] = bad_in ? 0LL : __double2ll_rn(__dmul_rn(x, 0x1p32));
+        const unsigned long long ab = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
+        mxb = ab > mxb ? ab : mxb;
+        V[b] = ab < 0x41d0000000000000ULL ? to_fixed(x) : 0LL; // below 2^30
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long ob = __shfl_xor_sync(FULL, mxb, o);
+        mxb = ob > mxb ? ob : mxb;
+    }
+    const bool bad_in = mxb >= 0x41d0000000000000ULL;
+    const double mx = bad_in ? 0.0 : __longlong_as_double((long long)mxb);
     // visited bits: the bins any walker of the window had visited when this launch started,
     // the start bin, and every bin this walker enters for the first time (always through the
     // float64 path below)
     // (replay has no window mask: every bin counts as visited there)
     const uint8_t *gmask = s.mask ? s.mask + (size_t)w * s.W : nullptr;
+#pragma unroll 4
     for (int i = 0; i < visw(s.W); ++i) { // word i: bins 32i .. 32i+31, one per lane
         const int b = 32 * i + lane;
         const unsigned bits = __ballot_sync(FULL, b < nb && (gmask == nullptr || gmask[b]));
@@ -432,11 +451,10 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
     }
     __syncwarp();
     if (lane == 0) vis[(kstart - lo) >> 5] |= 1u << ((kstart - lo) & 31); // the start bin
-    mx = warp_max(mx);
     // the shadow of a running window ends the launch below (max |ln g| + T ln f) 2^32 < 2^62,
     // and ln f 2^32 must not round to zero; a frozen window adds nothing to it
     const bool lnf_ok = frozen || (lnf >= 0x1p-32 && lnf < 0x1p20 && mx + (double)T * lnf < 0x1p30);
-    if (__any_sync(FULL, bad_in) || !lnf_ok) {
+    if (bad_in || !lnf_ok) {
         // the int64 shadow would overflow or lose the increment: leave the state untouched
         if (lane == 0) {
             if (AHEAD) store_relaxed(mem.ctl + 2, 1);
@@ -860,12 +878,11 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
     }
     if (!frozen) {
         double *gl = s.lng + (size_t)slot * s.W;
+        const ExactDiv by(lnfq);
+#pragma unroll 1
         for (int b = lane; b < nb; b += 32) {
-            const uint32_t v = visits(V, gl, b, lnfq);
-            if (v != 0u) {
-                gl[b] = seqadd(gl[b], lnf, v);
-                gH[b] += v;
-            }
+            const double x = gl[b];
+            write_back(gl, gH, b, lnf, x, by(V[b] - to_fixed(x)));
         }
     }
     nacc = __reduce_add_sync(FULL, nacc);
@@ -941,7 +958,7 @@ __device__ __forceinline__ void move_walker_thread(const State &s, const MoveCfg
         const double x = glng[b];
         bad = bad || !(fabs(x) < 0x1p30);
         mx = fmax(mx, fabs(x));
-        V[b] = bad ? 0LL : __double2ll_rn(__dmul_rn(x, 0x1p32));
+        V[b] = bad ? 0LL : to_fixed(x);
     }
     const bool lnf_ok = frozen || (lnf >= 0x1p-32 && lnf < 0x1p20 && mx + (double)T * lnf < 0x1p30);
     if (bad || !lnf_ok) {
@@ -1009,14 +1026,13 @@ __device__ __forceinline__ void move_walker_thread(const State &s, const MoveCfg
     } else {
         for (int i = 0; i < s.N; ++i) gsp[i] = sp[i];
     }
-    if (!frozen)
+    if (!frozen) {
+        const ExactDiv by(lnfq);
         for (int b = 0; b < nb; ++b) {
-            const uint32_t v = visits(V, glng, b, lnfq);
-            if (v != 0u) {
-                glng[b] = seqadd(glng[b], lnf, v);
-                gH[b] += v;
-            }
+            const double x = glng[b];
+            write_back(glng, gH, b, lnf, x, by(V[b] - to_fixed(x)));
         }
+    }
     s.k[slot] = k;
     s.step[slot] = st0 + (unsigned long long)T;
     s.acc[slot] += nacc;
