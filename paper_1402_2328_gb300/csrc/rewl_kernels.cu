@@ -83,9 +83,9 @@ cudaError_t launch_move(const State &s, const MoveCfg &c, cudaStream_t st)
 // ---------------------------------------------------------------------------------------
 // Seeded lattices and prep into the window: one warp per walker, the lattice in shared memory (a
 // 16-bit cell per site, the state in the low byte, a claim in the high one).  Far from the window a proposal is accepted by the sign of its
-// energy change alone, so a batch of 32 has no serial part but its conflicts (a site proposed
-// twice, or a neighbour that an earlier step of the batch changed: the batch ends there); near it
-// a prefix sum finds the step that reaches the window, and that step is decided by itself.
+// energy change alone, so a batch of 32 has no serial part but its conflicts (a site or a neighbour
+// that an earlier step of the batch changed: the batch ends there); near it a prefix sum finds the
+// step that reaches the window, and that step is decided by itself.
 // Bound by the latency of a batch.  Potts q=10 L=80, 1024 walkers, rewl_init with the lattices
 // and bins read back: 548 ms with one thread per walker on global memory, 7.7 ms with a warp each.
 // ---------------------------------------------------------------------------------------
@@ -149,32 +149,25 @@ __global__ void __launch_bounds__(128) k_init_prep(State s, long long prep_budge
             ++restarts;
         }
         const unsigned long long end = ps + budget;
+        // lane j's draw of step at + j; the next 32 are drawn while a batch waits for its lattice
+        auto draw = [&](unsigned long long at) {
+            const unsigned long long i = at + (unsigned long long)lane;
+            return philox((uint32_t)i, (uint32_t)(i >> 32), (uint32_t)(s.slot0 + slot), (s.inst << 8) | TAG_PREP,
+                          s.key0, s.key1);
+        };
+        u32x4 r = draw(ps);
         while (dist_to(k, lo, hi) > 0 && ps < end) {
             const int n = (int)min(32ULL, end - ps);
-            const unsigned long long i = ps + (unsigned long long)lane;
-            const u32x4 r = philox((uint32_t)i, (uint32_t)(i >> 32), (uint32_t)(s.slot0 + slot),
-                                   (s.inst << 8) | TAG_PREP, s.key0, s.key1);
             const int site = (int)mulhi(r.x, (uint32_t)N);
             int nl, nr, nu, nd;
             lat.nbrs(site, nl, nr, nu, nd);
             // claims: the lowest lane that proposes a site marks it
             if (lane < n) cellb[2 * site + 1] = (uint8_t)lane;
             __syncwarp();
-            unsigned own = cellb[2 * site + 1];
-            for (int it = 0; it < 32; ++it) { // each pass lowers some claim: ends within 32 passes
-                const bool again = lane < n && own > (unsigned)lane;
-                if (!__any_sync(FULL, again)) break;
-                if (again) cellb[2 * site + 1] = (uint8_t)lane;
-                __syncwarp();
-                own = cellb[2 * site + 1];
-                __syncwarp();
-            }
-            const bool dup = lane < n && own < (unsigned)lane;
-            const unsigned c1 = cell[nl], c2 = cell[nr], c3 = cell[nu], c4 = cell[nd];
-            const uint32_t s0 = cell[site] & 0xffu;
-            const unsigned claims = (shl_clamp(1u, c1 >> 8) | shl_clamp(1u, c2 >> 8) | shl_clamp(1u, c3 >> 8) |
-                                     shl_clamp(1u, c4 >> 8)) & below;
+            unsigned c0 = cell[site], c1 = cell[nl], c2 = cell[nr], c3 = cell[nu], c4 = cell[nd];
             const uint32_t nbytes = __byte_perm(__byte_perm(c1, c2, 0x0040), __byte_perm(c3, c4, 0x0040), 0x5410);
+            const uint32_t s0 = c0 & 0xffu;
+            const u32x4 rn = draw(ps + 32ULL);
             int snew, dk;
             if (ISING) {
                 snew = -(int)(int8_t)s0;
@@ -184,13 +177,36 @@ __global__ void __launch_bounds__(128) k_init_prep(State s, long long prep_budge
                 if (snew >= s.q) snew -= s.q;
                 dk = __popc(bytes_unequal<false>(nbytes, (uint32_t)snew)) - __popc(bytes_unequal<false>(nbytes, s0));
             }
+            bool dup = false; // an earlier lane proposes the same site
+            if (__any_sync(FULL, lane < n && (c0 >> 8) != (unsigned)lane)) {
+                unsigned own = c0 >> 8;
+                for (int it = 0; it < 32; ++it) { // each pass lowers some claim: ends within 32 passes
+                    const bool again = lane < n && own > (unsigned)lane;
+                    if (!__any_sync(FULL, again)) break;
+                    if (again) cellb[2 * site + 1] = (uint8_t)lane;
+                    __syncwarp();
+                    own = cellb[2 * site + 1];
+                    __syncwarp();
+                }
+                dup = lane < n && own < (unsigned)lane;
+                c0 = cell[site];
+                c1 = cell[nl];
+                c2 = cell[nr];
+                c3 = cell[nu];
+                c4 = cell[nd];
+            }
+            const unsigned claims = (shl_clamp(1u, c0 >> 8) | shl_clamp(1u, c1 >> 8) | shl_clamp(1u, c2 >> 8) |
+                                     shl_clamp(1u, c3 >> 8) | shl_clamp(1u, c4 >> 8)) & below;
             __syncwarp();
             if (lane < n) cellb[2 * site + 1] = (uint8_t)NO_CLAIM;
-            // accepted while the walker stays on its side of the window
+            // accepted while the walker stays on its side of the window.  The batch ends before a step whose
+            // site or neighbour an earlier accepted step proposes, and behind an accepted step whose
+            // claim an earlier lane holds (nobody else sees that one).
             const bool above = k > hi;
             bool acc = above ? dk <= 0 : dk >= 0;
             const unsigned accs = __ballot_sync(FULL, acc);
-            int done = (int)__reduce_min_sync(FULL, lane >= n || dup || (claims & accs) ? (unsigned)lane : 32u);
+            int done = (int)__reduce_min_sync(FULL, lane >= n || (claims & accs) ? (unsigned)lane
+                                                                                 : (dup && acc ? lane + 1u : 32u));
             const int d = acc && lane < done ? dk : 0;
             if (dist_to(k, lo, hi) > DM * 32) {
                 k += __reduce_add_sync(FULL, d);
@@ -216,6 +232,8 @@ __global__ void __launch_bounds__(128) k_init_prep(State s, long long prep_budge
             }
             if (lane < done && acc) cellb[2 * site] = (uint8_t)snew; // distinct sites
             ps += (unsigned long long)done;
+            if (done == 32) r = rn;
+            else r = draw(ps);
             __syncwarp();
         }
     }

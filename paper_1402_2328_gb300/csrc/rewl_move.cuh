@@ -629,11 +629,10 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
                 table_age = 0;
                 __syncwarp();
             }
-            // the step is surely accepted from bin offset x if D(x) > tS, surely rejected if
-            // D(x) < tR, whatever the visits since the table was taken did to ln g
+            // the step is accepted from bin offset x if D(x) > ln u; surely so, or surely rejected, if the
+            // two are further apart than mg, whatever the visits since the table was taken did to ln g
             const float mg = __fmaf_rn((float)(table_age + lane + 1), lnf_f, M);
-            const __half2 tS = __float2half2_rn(lnu + mg);
-            const float tR = lnu - mg;
+            const __half2 tS = __float2half2_rn(lnu);
             const uint4 *row = reinterpret_cast<const uint4 *>(tab + dkm * ROW_BYTES);
             const float *lrow = lin + dkm * LIN_ROW;
             unsigned S4[4]; // one a load, so that the chain is short
@@ -646,8 +645,8 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
                 for (int e = 0; e < 4; ++e)
                     S4[v] |= __hgt2_mask(*reinterpret_cast<const __half2 *>(&ww[e]), tS) & (0x00010001u << (4 * v + e));
             }
-            unsigned S = (S4[0] | S4[1]) | (S4[2] | S4[3]); // bit x: surely accepted from x
-            int known = 0; // -1: step `lane` was decided below
+            unsigned S = (S4[0] | S4[1]) | (S4[2] | S4[3]); // bit x: accepted from x, as far as the table tells
+            int mv;        // -1: step `lane` moves
             int4 d;        // of the lane's group of four steps: bin changes
             uint4 q;       // and masks: from bin offset x at the start of the group, step i of it
                            // moves if bit x of mask i is set, whatever the steps before it do
@@ -681,44 +680,56 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
                 yb += (sign_mask((int)(q.x << yb)) & g1) * d.x + (sign_mask((int)(q.y << yb)) & g2) * d.y +
                       (sign_mask((int)(q.z << yb)) & g3) * d.z;
                 xb = 31 - yb;
-                const int mv = sign_mask((int)(S << yb));
+                mv = sign_mask((int)(S << yb));
                 xa = xb + (mv & dk);
-                int sure = mv | known | sign_mask(__float_as_int(lrow[xb] - tR));
-                if (CHECK) sure = dz || (unsigned)(xb + dk - (lo - wbase)) >= (unsigned)nb ? -1 : 0;
-                stop_at(dz || mv != 0, sure);
+                // the table's verdict at xb: t < -mg rejected, t > mg accepted
+                const float t = lrow[xb] - lnu;
+                int ok = sign_mask(__float_as_int(__int_as_float(__float_as_int(t) ^ (mv & (int)0x80000000)) + mg));
+                if (CHECK) ok = dz || (unsigned)(xb + dk - (lo - wbase)) >= (unsigned)nb ? -1 : 0;
+                stop_at(dz || mv != 0, ok);
             };
             walk();
             bool fresh = table_age == 0;
             while (__builtin_expect(open, 0)) {
-                // step `stop`: its ln g difference with the visits before it, in float32
-                const int u = stop;
-                const int xu = __shfl_sync(FULL, xb, u), du = __shfl_sync(FULL, dk, u);
-                const int xt = xu + du;
-                if ((unsigned)xt >= 32u) {
-                    open = u == 0; // else the next batch's cache will hold the target
-                    break;
-                }
+                // Some step is too close for the table.  Every lane takes its own step's ln g
+                // difference with the visits on the path before it, in float32; the path is right as far
+                // as all of them agree with it.  The first one that does not is put right and the
+                // walk taken again.
                 if (!fresh) { // bring the cached values up to date
                     const float Mt = M;
                     cache_floats();
                     M = fmaxf(M, Mt);
                     fresh = true;
                 }
-                const unsigned bu = (1u << u) - 1u;
-                const int cx = __popc(__ballot_sync(FULL, xa == xu) & bu), ct = __popc(__ballot_sync(FULL, xa == xt) & bu);
-                const float e = __fmaf_rn((float)(cx - ct), lnf_f, __shfl_sync(FULL, Lw, xu) - __shfl_sync(FULL, Lw, xt)) -
-                                __shfl_sync(FULL, lnu, u);
+                const int xt = xb + dk;
+                unsigned at = below, to = below; // steps before this one that ended in xb, in xt
+#pragma unroll
+                for (int i = 0; i < 5; ++i) {
+                    const unsigned b = __ballot_sync(FULL, (xa >> i) & 1);
+                    at &= ((xb >> i) & 1) ? b : ~b;
+                    to &= ((xt >> i) & 1) ? b : ~b;
+                }
+                const bool out = (unsigned)xt >= 32u;
+                const float Lb = __shfl_sync(FULL, Lw, xb), Lt = __shfl_sync(FULL, Lw, xt);
+                const float e = out ? __int_as_float(0x7fc00000)
+                                    : __fmaf_rn((float)(__popc(at) - __popc(to)), lnf_f, Lb - Lt) - lnu;
                 if (CHECK) {
-                    const int sure = ((S >> xu) & 1u) ? 1 : (lrow[xu] < tR ? 0 : -1);
-                    scr = __shfl_sync(FULL, sure, u);
-                    if (scr < 0) scr = e > M ? 1 : (e < -M ? 0 : -1);
+                    const float t = lrow[xb] - lnu;
+                    const int v = t > mg ? 1 : (t < -mg ? 0 : (e > M ? 1 : (e < -M ? 0 : -1)));
+                    scr = __shfl_sync(FULL, v, stop);
+                    const int u_out = __shfl_sync(FULL, out ? 1 : 0, stop);
+                    open = stop == 0 || u_out == 0;
                     break;
                 }
-                if (!(fabsf(e) > M)) break; // too close: float64
-                if (lane == u) {
-                    known = -1;
-                    if (e > M) S |= 1u << xu;
+                stop_at(dz || mv != 0, dz || (mv ? e > M : e < -M) ? -1 : 0);
+                if (!open) break;
+                const int verdict = e > M ? 1 : (e < -M ? 0 : (out ? 2 : 3));
+                const int v = __shfl_sync(FULL, verdict, stop);
+                if (v >= 2) { // a target outside the cache: the next one will hold it; else float64
+                    open = stop == 0 || v == 3;
+                    break;
                 }
+                if (lane == stop) S = (S & ~(1u << xb)) | ((unsigned)v << xb);
                 walk();
             }
             table_age += stop;
