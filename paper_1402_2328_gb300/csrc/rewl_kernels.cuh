@@ -73,12 +73,17 @@ constexpr int MOVE_RING = 128;
 constexpr int MOVE_SCRATCH_BYTES = MOVE_TAB_BYTES + 9 * 36 * 4 + 24 * 16 + 32 * 4 + MOVE_RING * 20 + 16;
 // Largest ln f at which a batch is walked through the ratio table.  Above it the visits of the batch
 // itself leave too many steps undecided (us per launch, Potts L=80 64 x 16 and Ising L=64 32 x 16,
-// table / running walk: 522 / 638 and 440 / 455 at 2^-8, 632 / 639 and 556 / 454 at 2^-7).
-constexpr float TABLE_WALK_LNF = 0x1.8p-8f;
+// table / running walk: 532 / 564 and 427 / 446 at 2^-6, 590 / 565 and 474 / 448 at 2^-5).
+constexpr float TABLE_WALK_LNF = 0x1.8p-6f;
+// Largest ln f at which undecided steps are rare enough to be taken one by one: verifying the whole path
+// costs the walk registers (Potts L=40 at 2^-10: 490 us one by one, 474 verified, Ising L=64 at 2^-8 433
+// and 364; at 2^-14 L=8 .. 16 gain 2 % without, at 2^-12 the two are equal).
+constexpr float SURE_WALK_LNF = 0x1p-13f;
 // Growth of ln g (visits x ln f) after which the ratio table is taken anew: taking it costs about 300
-// cycles, a step left undecided twice that (us per launch at 2^-10 / 2^-6 / 2^-4: Ising L=32 8 x 8
-// at ln f = 2^-12 372 / 341 / 363, Ising L=8 whole run 1099 / 954 / 936).
-constexpr float TABLE_DRIFT = 0x1p-6f;
+// cycles, a step left undecided about as much verified and twice that one by one (us per launch at
+// 2^-10 / 2^-6 / 2^-4: Ising L=32 8 x 8 at ln f = 2^-12 372 / 341 / 363, Ising L=8 whole run 1099 / 954 /
+// 936; Potts L=40 at 2^-10, verified, 2^-6 / 2^-5: 485 / 474).
+constexpr float SURE_DRIFT = 0x1p-6f, VERIFIED_DRIFT = 0x1p-5f;
 // Cache offsets of the current bin between which the cached bins stay (8 .. 23: 1 % slower; a step
 // changes the bin by 4 at most).
 constexpr int CACHE_LO = 6, CACHE_HI = 25;

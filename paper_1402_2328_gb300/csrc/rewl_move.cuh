@@ -62,8 +62,9 @@ __device__ __forceinline__ int propose_dk(const int8_t *sp, const Lattice &lat, 
 //      surely accepted from x".  Walking the batch is then a chain of integer shifts and
 //      multiply-adds on these masks, four steps at a time.  A step that is surely accepted or
 //      rejected under a margin that covers every rounding and the visits since the table was
-//      taken needs no more; another one is decided in float32 with those visits, and if that
-//      is too close as well, on the shadow or in float64.
+//      taken needs no more; another one is decided in float32 with those visits (at middling
+//      ln f, where there are several, all lanes at once against the path just walked), and if
+//      that is too close as well, on the shadow or in float64.
 //      Large ln f, where each visit turns later decisions: the path is walked with running
 //      float32 values through shuffles, every step screened by the same kind of margin;
 //   4. the batch is cut before the first step whose site or a neighbour of it an earlier step of
@@ -82,9 +83,9 @@ __device__ __forceinline__ int propose_dk(const int8_t *sp, const Lattice &lat, 
 // round trips a batch that need no lattice, in a second warp while the walkers of the launch leave
 // warp slots free (move kernel, Ising L=64 32 x 16, ln f = 2^-20: 366 us with the drawing in the
 // same warp, 267 us with a second one; 600 us with the 32-step chain of shuffles, match_any and
-// predicates before).  Other workloads, us per launch of 10^4 moves, that kernel -> this one: Ising L=32
-// 8 x 8 at 2^-12 770 -> 341, Potts L=40 64 x 16 at 2^-10 810 -> 504, Potts L=80 64 x 16 at 2^-24
-// 700 -> 347, at ln f = 1 730 -> 638, Ising L=8 4 x 1 1960 -> 960.
+// predicates before).  Workloads, us per launch of 10^4 moves, that kernel -> this one: Ising L=64 32 x 16
+// at 2^-20 600 -> 261, Ising L=32 8 x 8 at 2^-12 770 -> 333, Potts L=40 64 x 16 at 2^-10 810 -> 474,
+// Potts L=80 64 x 16 at 2^-24 700 -> 335, at ln f = 1 730 -> 613, Ising L=8 4 x 1 1960 -> 920.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ double shadow_error(double maxabs, int T, double lnf, bool frozen)
 {
@@ -377,11 +378,14 @@ __device__ __forceinline__ void draw_walker(const State &s, const MoveCfg &c, co
     }
 }
 
+// How the batches of a launch are walked, by ln f: with running values; through the ratio table, the path
+// verified as a whole where a step is too close for it; through the table, such steps one by one.
+enum Walk { RUNNING, VERIFIED, SURE };
+
 // One walker's `c.T` moves; `base` is the walker's shared-memory block, the whole warp calls.
 // NP: pairs of steps in a batch (16, or fewer for small lattices, where sites soon repeat).
-// AHEAD: another warp draws the proposals (draw_walker), else this one does.  TABLE: the batches are
-// walked through the ratio table.
-template <bool ISING, bool REPLAY, bool CHECK, bool AHEAD, int NP, bool TABLE>
+// AHEAD: another warp draws the proposals (draw_walker), else this one does.
+template <bool ISING, bool REPLAY, bool CHECK, bool AHEAD, int NP, Walk WALK>
 __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, const int slot,
                                               unsigned char *base, const int lane)
 {
@@ -469,7 +473,7 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
     const float Mbase = (float)(c.eps_l + 2.0 * shadow_error(mx, T, lnf, frozen) * 0x1p-32) * (1.0f + 0x1p-20f) + 0x1p-21f;
     const float lnf_f = frozen ? 0.0f : (float)lnf;
     // visits after which the ratio table is taken anew
-    const int table_life = lnf_f > 0.0f ? (int)fminf(TABLE_DRIFT / lnf_f, 1e8f) : 100000000;
+    const int table_life = lnf_f > 0.0f ? (int)fminf((WALK == VERIFIED ? VERIFIED_DRIFT : SURE_DRIFT) / lnf_f, 1e8f) : 100000000;
 
     const unsigned long long st0 = s.step[slot];
     unsigned int nacc = 0, nex = 0, nmis = 0; // nacc: of this lane's steps
@@ -527,7 +531,7 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
         if (far) Lw = __int_as_float(0x7fc00000);
     };
     float *lin = mem.lin;
-    if (TABLE) { // row 0 of the table: a step that keeps the energy never moves
+    if (WALK != RUNNING) { // row 0 of the table: a step that keeps the energy never moves
         reinterpret_cast<__half *>(tab + DM * ROW_BYTES)[lane] = __float2half_rn(-INFINITY);
         lin[DM * LIN_ROW + lane] = -INFINITY;
     }
@@ -611,7 +615,7 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
             cache_store();
             cache_load(k);
         }
-        if (TABLE) {
+        if (WALK != RUNNING) {
             if (__builtin_expect(edge || table_age > table_life, 0)) { // rows of the ratio table
                 cache_floats();
 #pragma unroll
@@ -629,10 +633,12 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
                 table_age = 0;
                 __syncwarp();
             }
-            // the step is accepted from bin offset x if D(x) > ln u; surely so, or surely rejected, if the
-            // two are further apart than mg, whatever the visits since the table was taken did to ln g
+            // the step is surely accepted from bin offset x if D(x) > tA, surely rejected if
+            // D(x) < tR, whatever the visits since the table was taken did to ln g.  The walk takes
+            // what is not sure for a rejection (VERIFIED: for what the table says).
             const float mg = __fmaf_rn((float)(table_age + lane + 1), lnf_f, M);
-            const __half2 tS = __float2half2_rn(lnu);
+            const __half2 tS = __float2half2_rn(WALK == VERIFIED ? lnu : lnu + mg);
+            const float tR = lnu - mg, tA = lnu + mg;
             const uint4 *row = reinterpret_cast<const uint4 *>(tab + dkm * ROW_BYTES);
             const float *lrow = lin + dkm * LIN_ROW;
             unsigned S4[4]; // one a load, so that the chain is short
@@ -645,8 +651,8 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
                 for (int e = 0; e < 4; ++e)
                     S4[v] |= __hgt2_mask(*reinterpret_cast<const __half2 *>(&ww[e]), tS) & (0x00010001u << (4 * v + e));
             }
-            unsigned S = (S4[0] | S4[1]) | (S4[2] | S4[3]); // bit x: accepted from x, as far as the table tells
-            int mv;        // -1: step `lane` moves
+            unsigned S = (S4[0] | S4[1]) | (S4[2] | S4[3]); // bit x: accepted from x
+            int known = 0; // -1: step `lane` was decided below
             int4 d;        // of the lane's group of four steps: bin changes
             uint4 q;       // and masks: from bin offset x at the start of the group, step i of it
                            // moves if bit x of mask i is set, whatever the steps before it do
@@ -680,56 +686,92 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
                 yb += (sign_mask((int)(q.x << yb)) & g1) * d.x + (sign_mask((int)(q.y << yb)) & g2) * d.y +
                       (sign_mask((int)(q.z << yb)) & g3) * d.z;
                 xb = 31 - yb;
-                mv = sign_mask((int)(S << yb));
+                const int mv = sign_mask((int)(S << yb));
                 xa = xb + (mv & dk);
-                // the table's verdict at xb: t < -mg rejected, t > mg accepted
-                const float t = lrow[xb] - lnu;
-                int ok = sign_mask(__float_as_int(__int_as_float(__float_as_int(t) ^ (mv & (int)0x80000000)) + mg));
-                if (CHECK) ok = dz || (unsigned)(xb + dk - (lo - wbase)) >= (unsigned)nb ? -1 : 0;
-                stop_at(dz || mv != 0, ok);
+                int sure;
+                if (WALK == VERIFIED) {
+                    const float D = lrow[xb];
+                    sure = pick(mv, sign_mask(__float_as_int(tA - D)), sign_mask(__float_as_int(D - tR)));
+                } else {
+                    sure = mv | known | sign_mask(__float_as_int(lrow[xb] - tR));
+                }
+                if (CHECK) sure = dz || (unsigned)(xb + dk - (lo - wbase)) >= (unsigned)nb ? -1 : 0;
+                stop_at(dz || mv != 0, sure);
             };
             walk();
             bool fresh = table_age == 0;
             while (__builtin_expect(open, 0)) {
-                // Some step is too close for the table.  Every lane takes its own step's ln g
-                // difference with the visits on the path before it, in float32; the path is right as far
-                // as all of them agree with it.  The first one that does not is put right and the
-                // walk taken again.
-                if (!fresh) { // bring the cached values up to date
-                    const float Mt = M;
-                    cache_floats();
-                    M = fmaxf(M, Mt);
-                    fresh = true;
-                }
-                const int xt = xb + dk;
-                unsigned at = below, to = below; // steps before this one that ended in xb, in xt
+                if (WALK == VERIFIED) {
+                    if ((unsigned)__shfl_sync(FULL, xb + dk, stop) >= 32u) {
+                        open = stop == 0; // else the next batch's cache will hold the target
+                        break;
+                    }
+                    if (!fresh) { // bring the cached values up to date
+                        const float Mt = M;
+                        cache_floats();
+                        M = fmaxf(M, Mt);
+                        fresh = true;
+                    }
+                    // Some step is too close for the table.  Every lane takes its own step's ln g
+                    // difference with the visits on the path before it, in float32; the path is right
+                    // as far as all of them agree with it.  The first one that does not is put right
+                    // and the walk taken again.
+                    const int xt = xb + dk;
+                    unsigned at = below, to = below; // steps before this one that ended in xb, in xt
 #pragma unroll
-                for (int i = 0; i < 5; ++i) {
-                    const unsigned b = __ballot_sync(FULL, (xa >> i) & 1);
-                    at &= ((xb >> i) & 1) ? b : ~b;
-                    to &= ((xt >> i) & 1) ? b : ~b;
+                    for (int i = 0; i < 5; ++i) {
+                        const unsigned b = __ballot_sync(FULL, (xa >> i) & 1);
+                        at &= ((xb >> i) & 1) ? b : ~b;
+                        to &= ((xt >> i) & 1) ? b : ~b;
+                    }
+                    const bool out = (unsigned)xt >= 32u;
+                    const float Lb = __shfl_sync(FULL, Lw, xb), Lt = __shfl_sync(FULL, Lw, xt);
+                    const float e = out ? __int_as_float(0x7fc00000)
+                                        : __fmaf_rn((float)(__popc(at) - __popc(to)), lnf_f, Lb - Lt) - lnu;
+                    if (CHECK) {
+                        const float D = lrow[xb];
+                        scr = __shfl_sync(FULL, D > tA ? 1 : (D < tR ? 0 : (e > M ? 1 : (e < -M ? 0 : -1))), stop);
+                        break;
+                    }
+                    stop_at(dz || xa != xb, dz || (xa != xb ? e > M : e < -M) ? -1 : 0);
+                    if (!open) break;
+                    const int v = __shfl_sync(FULL, e > M ? 1 : (e < -M ? 0 : (out ? 2 : 3)), stop);
+                    if (v >= 2) { // outside the cache as above, or too close: float64
+                        open = stop == 0 || v == 3;
+                        break;
+                    }
+                    if (lane == stop) S = (S & ~(1u << xb)) | ((unsigned)v << xb);
+                } else {
+                    // step `stop`: its ln g difference with the visits before it, in float32
+                    const int u = stop;
+                    const int xu = __shfl_sync(FULL, xb, u), du = __shfl_sync(FULL, dk, u);
+                    const int xt = xu + du;
+                    if ((unsigned)xt >= 32u) {
+                        open = u == 0; // else the next batch's cache will hold the target
+                        break;
+                    }
+                    if (!fresh) { // bring the cached values up to date
+                        const float Mt = M;
+                        cache_floats();
+                        M = fmaxf(M, Mt);
+                        fresh = true;
+                    }
+                    const unsigned bu = (1u << u) - 1u;
+                    const int cx = __popc(__ballot_sync(FULL, xa == xu) & bu), ct = __popc(__ballot_sync(FULL, xa == xt) & bu);
+                    const float e = __fmaf_rn((float)(cx - ct), lnf_f, __shfl_sync(FULL, Lw, xu) - __shfl_sync(FULL, Lw, xt)) -
+                                    __shfl_sync(FULL, lnu, u);
+                    if (CHECK) {
+                        const int sure = ((S >> xu) & 1u) ? 1 : (lrow[xu] < tR ? 0 : -1);
+                        scr = __shfl_sync(FULL, sure, u);
+                        if (scr < 0) scr = e > M ? 1 : (e < -M ? 0 : -1);
+                        break;
+                    }
+                    if (!(fabsf(e) > M)) break; // too close: float64
+                    if (lane == u) {
+                        known = -1;
+                        if (e > M) S |= 1u << xu;
+                    }
                 }
-                const bool out = (unsigned)xt >= 32u;
-                const float Lb = __shfl_sync(FULL, Lw, xb), Lt = __shfl_sync(FULL, Lw, xt);
-                const float e = out ? __int_as_float(0x7fc00000)
-                                    : __fmaf_rn((float)(__popc(at) - __popc(to)), lnf_f, Lb - Lt) - lnu;
-                if (CHECK) {
-                    const float t = lrow[xb] - lnu;
-                    const int v = t > mg ? 1 : (t < -mg ? 0 : (e > M ? 1 : (e < -M ? 0 : -1)));
-                    scr = __shfl_sync(FULL, v, stop);
-                    const int u_out = __shfl_sync(FULL, out ? 1 : 0, stop);
-                    open = stop == 0 || u_out == 0;
-                    break;
-                }
-                stop_at(dz || mv != 0, dz || (mv ? e > M : e < -M) ? -1 : 0);
-                if (!open) break;
-                const int verdict = e > M ? 1 : (e < -M ? 0 : (out ? 2 : 3));
-                const int v = __shfl_sync(FULL, verdict, stop);
-                if (v >= 2) { // a target outside the cache: the next one will hold it; else float64
-                    open = stop == 0 || v == 3;
-                    break;
-                }
-                if (lane == stop) S = (S & ~(1u << xb)) | ((unsigned)v << xb);
                 walk();
             }
             table_age += stop;
@@ -912,11 +954,15 @@ __device__ __forceinline__ void move_walker(const State &s, const MoveCfg &c, co
 {
     if (s.status != nullptr && s.status->done) return;
     const int w = slot / s.m;
-    const bool table = s.finished[w] != 0 || s.lnf[w] <= (double)TABLE_WALK_LNF;
+    const double lnf = s.finished[w] ? 0.0 : s.lnf[w];
 #define REWL_WALK(NP)                                                                            \
     do {                                                                                         \
-        if (table) move_walker_n<ISING, REPLAY, CHECK, AHEAD, NP, true>(s, c, slot, base, lane); \
-        else move_walker_n<ISING, REPLAY, CHECK, AHEAD, NP, false>(s, c, slot, base, lane);      \
+        if (lnf <= (double)SURE_WALK_LNF)                                                        \
+            move_walker_n<ISING, REPLAY, CHECK, AHEAD, NP, SURE>(s, c, slot, base, lane);        \
+        else if (lnf <= (double)TABLE_WALK_LNF)                                                  \
+            move_walker_n<ISING, REPLAY, CHECK, AHEAD, NP, VERIFIED>(s, c, slot, base, lane);    \
+        else                                                                                     \
+            move_walker_n<ISING, REPLAY, CHECK, AHEAD, NP, RUNNING>(s, c, slot, base, lane);     \
     } while (0)
     if (s.N >= BATCH32_SITES) REWL_WALK(16);
     else if (s.N >= BATCH16_SITES) REWL_WALK(8);

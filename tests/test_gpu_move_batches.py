@@ -1,6 +1,6 @@
 """The move kernel's branches by size against the oracle, bit for bit: batches of 8, 16 and 32
-steps (lattices on both sides of each limit), the ratio-table walk and the running walk on both
-sides of the ln f that separates them, non-dyadic and frozen windows, and replay with rows so wide
+steps (lattices on both sides of each limit), the three kinds of walk on both sides of the ln f
+that separate them, non-dyadic and frozen windows, and replay with rows so wide
 that the batch scratch does not fit beside them."""
 import numpy as np
 import pytest
@@ -24,7 +24,8 @@ def cuda_lib():
 # lattices: 9 | 10 sites a side part batches of 8 and 16 steps, 21 | 22 those of 16 and 32
 @pytest.mark.parametrize("model,L", [(0, 9), (0, 10), (3, 9), (10, 10), (0, 21), (0, 22), (10, 21),
                                      (7, 22)])
-@pytest.mark.parametrize("lnf", [2.0 ** -7, 2.0 ** -8, 2.0 ** -8 * 1.01, 3e-5, 2.0 ** -26])
+@pytest.mark.parametrize("lnf", [2.0 ** -5, 1.5 * 2.0 ** -6, 2.0 ** -7, 2.0 ** -8 * 1.01, 2.0 ** -12,
+                                 2.0 ** -13, 3e-5, 2.0 ** -26])
 def test_batch_sizes_and_walks_bit_exact(model, L, lnf):
     g, o = _pair(model, L, 2, 2, lnf_final=1e-9, seed=I.seed_for(7, L + model), interval=1777,
                  lnf_init=1.0)
