@@ -306,7 +306,7 @@ __device__ __forceinline__ void check_window(const State &s, const int w, const 
         unsigned long long sum = 0;
         uint32_t mn = 0xffffffffu;
         int cnt = 0;
-#pragma unroll 4
+#pragma unroll 8
         for (int b = lane; b < nb; b += 32) { // both loads unconditional: they overlap
             const uint32_t v = H[b];
             if (mask[b]) {

@@ -85,7 +85,7 @@ __device__ __forceinline__ int propose_dk(const int8_t *sp, const Lattice &lat, 
 // same warp, 267 us with a second one; 600 us with the 32-step chain of shuffles, match_any and
 // predicates before).  Workloads, us per launch of 10^4 moves, that kernel -> this one: Ising L=64 32 x 16
 // at 2^-20 600 -> 261, Ising L=32 8 x 8 at 2^-12 770 -> 333, Potts L=40 64 x 16 at 2^-10 810 -> 474,
-// Potts L=80 64 x 16 at 2^-24 700 -> 335, at ln f = 1 730 -> 613, Ising L=8 4 x 1 1960 -> 920.
+// Potts L=80 64 x 16 at 2^-24 700 -> 333, at ln f = 1 730 -> 584, Ising L=8 4 x 1 1960 -> 911.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ double shadow_error(double maxabs, int T, double lnf, bool frozen)
 {
@@ -784,16 +784,25 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
             // v = M - (ln g(k) - ln g(k') - ln u); accept if v < 0, reject if v > 2M, else unsure.
             // A target outside the 32 cached bins reads a wrong lane; such steps are found after
             // the loop and cut there as well.
+            // Steps that keep the energy never move: only the others are walked, each with the ln f of
+            // the visits such steps made since the one before it (G).
             cache_floats();
-            const float thr = dz ? INFINITY : lnu;
-            reinterpret_cast<uint2 *>(bc)[lane] = make_uint2(__float_as_uint(thr + M), (unsigned)dk);
+            const unsigned act = __ballot_sync(FULL, !dz && lane < n), earlier = act & below;
+            const int rank = __popc(earlier), nact = __popc(act);
+            float2 *gap = reinterpret_cast<float2 *>(bc + 16);
+            if (!dz) {
+                reinterpret_cast<uint2 *>(bc)[rank] = make_uint2(__float_as_uint(lnu + M), (unsigned)dk);
+                reinterpret_cast<float *>(gap)[rank] = (float)(lane - 32 + __clz(earlier)) * lnf_f;
+            }
             __syncwarp();
             float Lr = Lw;   // the cache, with the running values of the bins left
             int xk = x;      // cache offset of the current bin
             float Lk = 0.0f; // its running value (the cache holds it only once left)
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
+                if ((p & 1) == 0 && p > 0 && 2 * p >= nact) break; // (what is behind nact is not read)
                 const uint4 a = bc[p];
+                const float2 G = gap[p];
                 const int d0 = (int)a.y, d1 = (int)a.w;
                 const int x0 = xk + d0; // k' of step i
                 const int xA = x0 + d1; // k' of step i+1 if step i moved
@@ -801,10 +810,12 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
                 const float L0 = __shfl_sync(FULL, Lr, x0);
                 const float LA_ = __shfl_sync(FULL, Lr, xA);
                 const float LR = __shfl_sync(FULL, Lr, xR);
+                Lk += G.x;
                 const float LA = (d1 == -d0) ? Lk : LA_; // back to the bin just left
                 const int onk = lane == xk ? -1 : 0, on0 = lane == x0 ? -1 : 0;
-                const float Ls = Lk + lnf_f; // value after step i if stayed
-                const float Lm = L0 + lnf_f; // value after step i if moved
+                const float G1 = lnf_f + G.y;  // step i's visit and those before step i+1
+                const float Ls = Lk + G1;      // value before step i+1 if step i stayed
+                const float Lm = L0 + G1;      // value before step i+1 if step i moved
                 const float v0 = (__uint_as_float(a.x) - Lk) + L0;
                 const int m0 = sign_mask(__float_as_int(v0));
                 const float v1 = pickf(m0, (__uint_as_float(a.z) - Lm) + LA, (__uint_as_float(a.z) - Ls) + LR);
@@ -819,14 +830,14 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
                     trail[p] = make_uint4((unsigned)xc, __float_as_uint(v0), (unsigned)xk, __float_as_uint(v1));
             }
             __syncwarp();
-            const uint2 tr = reinterpret_cast<const uint2 *>(trail)[lane];
-            xa = (int)tr.x;
+            const uint2 *walked = reinterpret_cast<const uint2 *>(trail);
+            xb = rank ? (int)walked[rank - 1].x : x;
+            const uint2 tr = walked[rank & 31];
+            xa = dz ? xb : (int)tr.x;
             const float v = __uint_as_float(tr.y);
-            const int xup = __shfl_up_sync(FULL, xa, 1);
-            xb = lane == 0 ? x : xup;
             const bool oob = (unsigned)(xb + dk) >= 32u;
             const float M2 = 2.0f * M * (1.0f + 0x1p-20f);
-            bool ok = (v < 0.0f || v > M2) && !oob;
+            bool ok = dz || ((v < 0.0f || v > M2) && !oob);
             if (CHECK) ok = dz || (unsigned)(xb + dk - (lo - wbase)) >= (unsigned)nb;
             stop_at(dz || xa != xb, ok ? -1 : 0);
             if (open) {
