@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "rewl_device.cuh"
+#include "rewl_em.cuh"
 #include "rewl_handle.h"
 
 using namespace rewl;
@@ -34,14 +35,7 @@ __global__ void k_measure_em(State s)
     if (s.status->done) return;
     const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (warp >= s.nw) return; // uniform per warp
-    const int8_t *sp = s.spins + (size_t)s.cfg[warp] * s.spin_stride;
-    unsigned up = 0;
-    for (int i = lane; i < s.N; i += 32) up += sp[i] > 0 ? 1u : 0u;
-    up = __reduce_add_sync(0xffffffffu, up);
-    if (lane == 0) {
-        const int w = warp / s.m;
-        atomicAdd(&s.hem[((size_t)w * s.W + (size_t)(s.k[warp] - s.lo[w])) * (size_t)(s.N + 1) + up], 1u);
-    }
+    measure_walker(s, warp, warp / s.m, lane);
 }
 
 __device__ unsigned long long block_sum_u64(unsigned long long v)
@@ -321,7 +315,7 @@ cudaError_t join_core(const double *S, const int *d_lo, const int *d_hi, int h, 
 namespace rewl {
 cudaError_t launch_measure_em(const State &s, cudaStream_t st)
 {
-    if (!s.hem) return cudaSuccess;
+    if (!s.hem || measured_in_tail(s)) return cudaSuccess;
     const int threads = 256, blocks = (s.nw * 32 + threads - 1) / threads;
     k_measure_em<<<blocks, threads, 0, st>>>(s);
     return cudaGetLastError();

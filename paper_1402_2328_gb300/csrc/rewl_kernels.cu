@@ -14,6 +14,7 @@
 #include <cstdint>
 
 #include "rewl_device.cuh"
+#include "rewl_em.cuh"
 #include "rewl_kernels.cuh"
 #include "rewl_move.cuh"
 
@@ -87,7 +88,7 @@ cudaError_t launch_move(const State &s, const MoveCfg &c, cudaStream_t st)
 // that an earlier step of the batch changed: the batch ends there); near it a prefix sum finds the
 // step that reaches the window, and that step is decided by itself.
 // Bound by the latency of a batch.  Potts q=10 L=80, 1024 walkers, rewl_init with the lattices
-// and bins read back: 548 ms with one thread per walker on global memory, 7.7 ms with a warp each.
+// and bins read back: 548 ms with one thread per walker on global memory, 6.8 ms with a warp each.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ int dist_to(int k, int lo, int hi)
 {
@@ -459,10 +460,13 @@ __device__ __forceinline__ unsigned arrive(unsigned *counter)
 
 // Window w's part of the end of a round.  s.sync: one counter per pair of the round, then one for
 // the windows; all zero between launches.
-__device__ __forceinline__ void round_tail(const State &s, const int w, const double flatness, const double lnf_final)
+__device__ __forceinline__ void round_tail(const State &s, const int w, const double flatness, const double lnf_final,
+                                           const bool measure)
 {
     if (s.status->done) return;
     const long long rd = s.status->round;
+    if (measure) // before the arrival below, after which configurations move
+        for (int i = threadIdx.x >> 5; i < s.m; i += blockDim.x >> 5) measure_walker(s, w * s.m + i, w, threadIdx.x & 31);
     check_window(s, w, flatness, lnf_final);
     // pairs (a, a+1) with the global window index w0 + a of the parity of the round
     const int a = ((w + s.w0 - rd) & 1) == 0 ? w : w - 1;
@@ -487,7 +491,7 @@ __device__ __forceinline__ void round_tail(const State &s, const int w, const do
 
 __global__ void __launch_bounds__(512) k_round_tail(State s, double flatness, double lnf_final)
 {
-    round_tail(s, blockIdx.x, flatness, lnf_final);
+    round_tail(s, blockIdx.x, flatness, lnf_final, measured_in_tail(s));
 }
 
 // tab[b] = (instance, window); prm[instance] = (flatness, ln f_final)
@@ -498,7 +502,7 @@ __global__ void __launch_bounds__(512) k_round_tail_batch(const State *__restric
     const int2 t = tab[blockIdx.x];
     const State s = states[t.x];
     const double2 p = prm[t.x];
-    round_tail(s, t.y, p.x, p.y);
+    round_tail(s, t.y, p.x, p.y, false);
 }
 
 cudaError_t launch_round_tail_batch(const State *states, const int2 *tab, int n, const double2 *prm,

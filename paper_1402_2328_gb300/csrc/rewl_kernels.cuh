@@ -73,7 +73,7 @@ constexpr int MOVE_RING = 128;
 constexpr int MOVE_SCRATCH_BYTES = MOVE_TAB_BYTES + 9 * 36 * 4 + 24 * 16 + 32 * 4 + MOVE_RING * 20 + 16;
 // Largest ln f at which a batch is walked through the ratio table.  Above it the visits of the batch
 // itself leave too many steps undecided (us per launch, Potts L=80 64 x 16 and Ising L=64 32 x 16,
-// table / running walk: 532 / 564 and 427 / 446 at 2^-6, 590 / 565 and 474 / 448 at 2^-5).
+// table / running walk: 535 / 551 and 430 / 429 at 2^-6, 594 / 553 and 480 / 429 at 2^-5).
 constexpr float TABLE_WALK_LNF = 0x1.8p-6f;
 // Largest ln f at which undecided steps are rare enough to be taken one by one: verifying the whole path
 // costs the walk registers (Potts L=40 at 2^-10: 490 us one by one, 474 verified, Ising L=64 at 2^-8 433
