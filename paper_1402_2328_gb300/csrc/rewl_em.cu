@@ -28,6 +28,7 @@ using namespace rewl;
 namespace {
 
 constexpr int EM_THREADS = 256;
+constexpr int EM_SUMS = 1024; // partial sums of the norm, at most
 constexpr double EM_LN2 = 0x1.62e42fefa39efp-1;
 
 __global__ void k_measure_em(State s)
@@ -148,37 +149,65 @@ __global__ void k_join_cand(const double *__restrict__ S, const int *__restrict_
     if (threadIdx.x == 0) part[(size_t)p * gridDim.x + blockIdx.x] = sh[0];
 }
 
-// one thread: join points and the chain of shifts (shift of window w+1 from the already
-// shifted window w)
-__global__ void k_join_finish(const double *__restrict__ S, const int *__restrict__ lo,
-                              const int *__restrict__ hi, int h, int W, int N1, int nblk,
-                              const Best *__restrict__ part, double *shift, int *joins, int *ok)
+// One CTA: join points, a warp per pair, and the chain of shifts by one thread (shift of window
+// w+1 from the already shifted window w).  at: the two fragments' values at the join, per pair.
+// The scan of the candidates by one thread took 60 us for 3 pairs of 112, this 7.
+__global__ void __launch_bounds__(EM_THREADS)
+    k_join_finish(const double *__restrict__ S, const int *__restrict__ lo, const int *__restrict__ hi, int h, int W,
+                  int N1, int nblk, const Best *__restrict__ part, double2 *at, double *shift, int *joins, int *ok,
+                  unsigned *arrived)
 {
-    shift[0] = 0.0;
-    *ok = 0;
-    for (int p = 0; p + 1 < h; ++p) {
+    const int lane = threadIdx.x & 31;
+    int bad = 0;
+    for (int p = threadIdx.x >> 5; p + 1 < h; p += EM_THREADS / 32) {
         Best b{-INFINITY, LLONG_MAX, LLONG_MAX};
-        for (int i = 0; i < nblk; ++i) b = better(b, part[(size_t)p * nblk + i]);
+        for (int i = lane; i < nblk; i += 32) b = better(b, part[(size_t)p * nblk + i]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            b = better(b, Best{__shfl_xor_sync(0xffffffffu, b.dot, o), __shfl_xor_sync(0xffffffffu, b.t, o),
+                               __shfl_xor_sync(0xffffffffu, b.fb, o)});
         const long long npts = (long long)(hi[p] - lo[p + 1] + 1) * N1;
-        long long t;
-        if (b.t != LLONG_MAX) t = b.t;
-        else if (b.fb != LLONG_MAX) t = b.fb % npts;
-        else return;
-        const int k = lo[p + 1] + (int)(t / N1), j = (int)(t % N1);
-        const double va = S[((size_t)p * W + (k - lo[p])) * N1 + j];
-        const double vb = S[((size_t)(p + 1) * W + (k - lo[p + 1])) * N1 + j];
-        shift[p + 1] = __dsub_rn(__dadd_rn(va, shift[p]), vb);
-        joins[2 * p] = k;
-        joins[2 * p + 1] = j;
+        const long long t = b.t != LLONG_MAX ? b.t : b.fb != LLONG_MAX ? b.fb % npts : -1;
+        if (t < 0) bad = 1; // no point in common
+        if (t >= 0 && lane == 0) {
+            const int k = lo[p + 1] + (int)(t / N1), j = (int)(t % N1);
+            at[p] = make_double2(S[((size_t)p * W + (k - lo[p])) * N1 + j],
+                                 S[((size_t)(p + 1) * W + (k - lo[p + 1])) * N1 + j]);
+            joins[2 * p] = k;
+            joins[2 * p + 1] = j;
+        }
     }
-    *ok = 1;
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x != 0) return;
+    *ok = !bad;
+    *arrived = 0u;
+    double sh = 0.0;
+    shift[0] = sh;
+    for (int p = 0; p + 1 < h; ++p) {
+        if (!bad) sh = __dsub_rn(__dadd_rn(at[p].x, sh), at[p].y);
+        shift[p + 1] = sh;
+    }
 }
 
-// Eq. (4), windows merged in order at every point
+// largest value of a CTA (NaN aside), to all threads
+__device__ double block_max(double v)
+{
+    __shared__ double sh[EM_THREADS];
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = EM_THREADS / 2; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + o]);
+        __syncthreads();
+    }
+    return sh[0];
+}
+
+// Eq. (4), windows merged in order at every point; and each CTA's largest value
 __global__ void k_combine_em(const double *__restrict__ S, const int *__restrict__ lo,
                              const int *__restrict__ hi, int h, int W, int N1, long long n,
-                             const double *__restrict__ shift, double *__restrict__ out)
+                             const double *__restrict__ shift, double *__restrict__ out, double *part_max)
 {
+    double m = -INFINITY;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
          t += (long long)gridDim.x * blockDim.x) {
         const int k = (int)(t / N1), j = (int)(t % N1);
@@ -196,32 +225,25 @@ __global__ void k_combine_em(const double *__restrict__ S, const int *__restrict
             }
         }
         out[t] = o;
+        m = fmax(m, o);
     }
+    m = block_max(m);
+    if (threadIdx.x == 0) part_max[blockIdx.x] = m;
 }
 
-// normalisation: block maxima, then block sums of exp(out - max), then the shift
-__global__ void k_em_max(const double *__restrict__ x, long long n, double *part)
+// Normalisation: sums of exp(out - max) per CTA; the last CTA to come adds them up in order, and its
+// log of the norm is what the next launch subtracts.  (The partial results read one after the other by
+// every thread of both launches, and the maxima in a launch of their own: 133 us for 66,049 points, now
+// 22.)
+__global__ void __launch_bounds__(EM_THREADS)
+    k_em_sumexp(const double *__restrict__ x, long long n, const double *__restrict__ part_max, int nmax,
+                double *part, double target, double *norm, unsigned *arrived)
 {
-    __shared__ double sh[EM_THREADS];
-    double m = -INFINITY;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x)
-        m = fmax(m, x[t]);
-    sh[threadIdx.x] = m;
-    __syncthreads();
-    for (int o = EM_THREADS / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + o]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
-
-__global__ void k_em_sumexp(const double *__restrict__ x, long long n, const double *part_max,
-                            int nblk, double *part)
-{
-    __shared__ double sh[EM_THREADS];
+    __shared__ double sh[EM_SUMS];
+    __shared__ bool last;
     double mx = -INFINITY;
-    for (int i = 0; i < nblk; ++i) mx = fmax(mx, part_max[i]);
+    for (int i = threadIdx.x; i < nmax; i += EM_THREADS) mx = fmax(mx, part_max[i]);
+    mx = block_max(mx);
     double s = 0.0;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
          t += (long long)gridDim.x * blockDim.x)
@@ -232,16 +254,26 @@ __global__ void k_em_sumexp(const double *__restrict__ x, long long n, const dou
         if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = sh[0];
+        __threadfence();
+        last = atomicAdd(arrived, 1u) == gridDim.x - 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += EM_THREADS) sh[i] = __ldcg(part + i);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    s = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < (int)gridDim.x; ++i) s += sh[i];
+    *norm = (mx + log(s)) - target;
 }
 
-__global__ void k_em_shift(double *x, long long n, const double *part_max, const double *part_sum,
-                           int nblk, double target)
+__global__ void k_em_shift(double *x, long long n, const double *__restrict__ norm)
 {
-    double mx = -INFINITY, s = 0.0;
-    for (int i = 0; i < nblk; ++i) mx = fmax(mx, part_max[i]);
-    for (int i = 0; i < nblk; ++i) s += part_sum[i];
-    const double c = (mx + log(s)) - target;
+    const double c = *norm;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n;
          t += (long long)gridDim.x * blockDim.x)
         if (x[t] > -INFINITY) x[t] -= c;
@@ -260,53 +292,52 @@ template <class T> T *em_alloc(size_t n, cudaError_t &e)
     return p;
 }
 
-// the join on device fragments S [h][W][N1]; lo/hi device; out device (B+1) x N1
-cudaError_t join_core(const double *S, const int *d_lo, const int *d_hi, int h, int W, int B, int N1,
-                      double de, double dq, double target, double *out, int *joins_host, int *ok_host,
-                      cudaStream_t st)
+// the join on device fragments S [h][W][N1]; lo/hi on the device, and on the host; out device (B+1) x N1
+cudaError_t join_core(const double *S, const int *d_lo, const int *d_hi, const int *lo, const int *hi, int h, int W,
+                      int B, int N1, double de, double dq, double target, double *out, int *joins_host,
+                      int *ok_host, cudaStream_t st)
 {
     cudaError_t e = cudaSuccess;
     const int pairs = std::max(h - 1, 0);
     long long maxpts = 0;
-    std::vector<int> lo(h), hi(h);
-    e = cudaMemcpyAsync(lo.data(), d_lo, h * sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hi.data(), d_hi, h * sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return e;
     for (int p = 0; p < pairs; ++p) maxpts = std::max(maxpts, (long long)(hi[p] - lo[p + 1] + 1) * N1);
     const int nblk = grid_for(maxpts, 128);
-    Best *part = em_alloc<Best>((size_t)std::max(pairs, 1) * nblk, e);
-    double *shift = em_alloc<double>(h, e);
-    int *joins = em_alloc<int>(2 * (size_t)std::max(pairs, 1), e);
-    int *ok = em_alloc<int>(1, e);
     const long long n = (long long)(B + 1) * N1;
-    const int nred = grid_for(n, 1024);
-    double *pmax = em_alloc<double>(nred, e), *psum = em_alloc<double>(nred, e);
-    if (e == cudaSuccess && pairs > 0) {
+    const int nred = grid_for(n, EM_SUMS), ncomb = grid_for(n, 4096);
+    // one allocation: at [pairs], part [pairs][nblk], shift [h], maxima, sums, norm, joins, ok, arrivals
+    const size_t np1 = std::max(pairs, 1);
+    const size_t bytes = np1 * sizeof(double2) + np1 * nblk * sizeof(Best) +
+                         ((size_t)h + ncomb + nred + 1) * sizeof(double) + (2 * np1 + 2) * sizeof(int);
+    char *ws = em_alloc<char>(bytes, e);
+    if (e != cudaSuccess) return e;
+    double2 *at = reinterpret_cast<double2 *>(ws);
+    Best *part = reinterpret_cast<Best *>(at + np1);
+    double *shift = reinterpret_cast<double *>(part + np1 * nblk), *pmax = shift + h, *psum = pmax + ncomb,
+           *norm = psum + nred;
+    int *joins = reinterpret_cast<int *>(norm + 1), *ok = joins + 2 * np1;
+    unsigned *arrived = reinterpret_cast<unsigned *>(ok + 1);
+    if (pairs > 0) {
         k_join_cand<<<dim3(nblk, pairs), EM_THREADS, 0, st>>>(S, d_lo, d_hi, W, N1, de, dq, part);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        k_join_finish<<<1, 1, 0, st>>>(S, d_lo, d_hi, h, W, N1, nblk, part, shift, joins, ok);
+        k_join_finish<<<1, EM_THREADS, 0, st>>>(S, d_lo, d_hi, h, W, N1, nblk, part, at, shift, joins, ok, arrived);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        k_combine_em<<<grid_for(n, 4096), EM_THREADS, 0, st>>>(S, d_lo, d_hi, h, W, N1, n, shift, out);
+        k_combine_em<<<ncomb, EM_THREADS, 0, st>>>(S, d_lo, d_hi, h, W, N1, n, shift, out, pmax);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        k_em_max<<<nred, EM_THREADS, 0, st>>>(out, n, pmax);
-        k_em_sumexp<<<nred, EM_THREADS, 0, st>>>(out, n, pmax, nred, psum);
-        k_em_shift<<<grid_for(n, 4096), EM_THREADS, 0, st>>>(out, n, pmax, psum, nred, target);
+        k_em_sumexp<<<nred, EM_THREADS, 0, st>>>(out, n, pmax, ncomb, psum, target, norm, arrived);
+        k_em_shift<<<grid_for(n, 4096), EM_THREADS, 0, st>>>(out, n, norm);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(ok_host, ok, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess && joins_host && pairs > 0)
         e = cudaMemcpyAsync(joins_host, joins, 2 * (size_t)pairs * sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    void *ptrs[] = {part, shift, joins, ok, pmax, psum};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
+    cudaFree(ws);
     return e;
 }
 
@@ -360,7 +391,8 @@ int rewl_join_em(const double *S, int h, int W, int B, int N1, const int *lo_hi,
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_lohi, lo_hi, 2 * (size_t)h * sizeof(int), cudaMemcpyHostToDevice, st);
     int ok = 0;
     if (e == cudaSuccess)
-        e = join_core(S, d_lohi, d_lohi + h, h, W, B, N1, de, dq, norm_target, out, joins, &ok, st);
+        e = join_core(S, d_lohi, d_lohi + h, lo_hi, lo_hi + h, h, W, B, N1, de, dq, norm_target, out, joins, &ok,
+                      st);
     if (d_lohi) cudaFree(d_lohi);
     if (e != cudaSuccess) {
         g_err = std::string("rewl_join_em: ") + cudaGetErrorString(e);
@@ -390,7 +422,7 @@ int rewl_stitch_em(rewl_t r, double *out, size_t n, int *joins)
     }
     int ok = 0;
     if (e == cudaSuccess)
-        e = join_core(S, r->st.lo, r->st.hi, r->h, r->W, r->B, N1, 4.0, 2.0,
+        e = join_core(S, r->st.lo, r->st.hi, r->lo.data(), r->hi.data(), r->h, r->W, r->B, N1, 4.0, 2.0,
                       (double)r->N * std::log(2.0), d_out, joins, &ok, r->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, d_out, npts * 8, cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);

@@ -29,3 +29,35 @@ def test_measurement_routes_bit_exact(L, h, m):
     for f in ("spins", "k", "lng", "H"):
         assert np.array_equal(a[f], b[f]), f
     g.close()
+
+
+# one window, fewer and more pairs than the CTA that picks the join points has warps, fewer and more points
+# than it has partial sums for (1024 x 256).  The norm: a sum of n <= 4e5 positive terms of 2^-53 relative
+# rounding each, far below 1e-11 of ln g.
+@pytest.mark.parametrize("B,N1,h", [(12, 2, 1), (36, 9, 3), (300, 5, 40), (64, 700, 2), (401, 1001, 9)])
+def test_join_em_sizes(B, N1, h):
+    import torch
+    import oracle as O
+    import paper_1402_2328_gb300.rewl as R
+    lo, hi = O.windows(B, h, 0.75)
+    W = int((hi - lo).max()) + 1
+    rng = np.random.default_rng(B)
+    kk, jj = np.meshgrid(np.arange(B + 1) / B, np.arange(N1) / N1, indexing="ij")
+    base = 40 * np.sin(2.1 * kk + 0.3) * np.cos(1.3 * jj - 0.2) + 9 * kk * jj
+    S = np.full((h, W, N1), -np.inf)
+    for w in range(h):
+        S[w, : hi[w] - lo[w] + 1] = base[lo[w]: hi[w] + 1] + rng.normal(0, 10) + rng.normal(
+            0, 1e-3, (hi[w] - lo[w] + 1, N1))
+    S[rng.random(S.shape) < 0.05] = -np.inf
+    ref, jref = O.join_em(lo, hi, S, B, N1 - 1)
+    out = torch.zeros((B + 1, N1), dtype=torch.float64, device="cuda")
+    joins = R.join_em(torch.from_numpy(S).cuda(), lo, hi, B, out)
+    a = out.cpu().numpy()
+    assert np.array_equal(joins, jref)
+    fin = np.isfinite(ref)
+    assert np.array_equal(np.isfinite(a), fin)
+    assert np.max(np.abs(a[fin] - ref[fin])) <= 1e-11 * max(1.0, np.max(np.abs(ref[fin])))
+    if h > 1:  # the last two windows share no point: refused
+        S[h - 1, : hi[h - 2] - lo[h - 1] + 1] = -np.inf
+        with pytest.raises(R.REWLError):
+            R.join_em(torch.from_numpy(S).cuda(), lo, hi, B, out)
