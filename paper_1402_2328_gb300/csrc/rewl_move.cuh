@@ -354,7 +354,10 @@ __device__ __forceinline__ void store_relaxed(int *p, int v)
     asm volatile("st.relaxed.cta.shared.b32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
 }
 
-constexpr int SPIN_LIMIT = 1 << 22; // polls of shared memory before a warp gives up on its partner
+// Polls of shared memory before a warp gives up on its partner: the first warp on the second, which
+// is never long, and the second, asleep between polls, on the first, which may rebuild float64
+// values for seconds (a tie in every addition of a bin's 10^8 visits).
+constexpr int SPIN_LIMIT = 1 << 22, SLEEP_LIMIT = 1 << 28;
 
 // The second warp of a walker: draws blocks ahead of the first as the ring has room.
 template <bool ISING>
@@ -369,7 +372,7 @@ __device__ __forceinline__ void draw_walker(const State &s, const MoveCfg &c, co
     Drawn before;
     for (int g = 0; g < c.T + 64; g += 32) { // the first warp asks for 33 steps beyond the last
         for (int it = 0; g + 32 - load_acquire(mem.ctl + 1) > MOVE_RING; ++it) {
-            if (load_acquire(mem.ctl + 2) || it > SPIN_LIMIT) return;
+            if (load_acquire(mem.ctl + 2) || it > SLEEP_LIMIT) return;
             __nanosleep(50);
         }
         draw_block<ISING, false>(s, c, mem, slot, st0, g, before, lane);
