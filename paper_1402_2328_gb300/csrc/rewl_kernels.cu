@@ -816,26 +816,12 @@ __device__ double block_reduce_sum(double v)
     return v;
 }
 
-// (value, key) pairs: the smaller value, ties -> the smaller key; over the warp, every lane gets it
-__device__ __forceinline__ void warp_argmin(double &v, int &key)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(FULL, v, o);
-        const int ok = __shfl_xor_sync(FULL, key, o);
-        if (ov < v || (ov == v && ok < key)) {
-            v = ov;
-            key = ok;
-        }
-    }
-}
-
-// Join bin of windows (w, w+1) behind bin `prev`, by one warp: argmin |beta_w - beta_(w+1)| by the
+// Join bin of windows (w, w+1) behind bin `prev`, by the whole CTA: argmin |beta_w - beta_(w+1)| by the
 // 5-point stencil, else the 3-point one, else the bin valid in both nearest the overlap's midpoint;
 // ties -> smaller bin; -1: none.
 __device__ int join_bin(const State &s, const double *mean, int w, int prev, double de, int step)
 {
-    const int W = s.W, lane = threadIdx.x & 31;
+    const int W = s.W, first = threadIdx.x, by = blockDim.x;
     const double *la = mean + (size_t)w * W, *lb = mean + (size_t)(w + 1) * W;
     const uint8_t *va = s.mask + (size_t)w * W, *vb = s.mask + (size_t)(w + 1) * W;
     const int loa = s.lo[w], hia = s.hi[w], lob = s.lo[w + 1], hib = s.hi[w + 1];
@@ -843,7 +829,7 @@ __device__ int join_bin(const State &s, const double *mean, int w, int prev, dou
     for (int npts = 5; npts >= 3; npts -= 2) {
         double best = INFINITY;
         int bk = 0x7fffffff;
-        for (int k = max(lob, prev + 1) + lane; k <= hia; k += 32) {
+        for (int k = max(lob, prev + 1) + first; k <= hia; k += by) {
             if (!va[k - loa] || !vb[k - lob]) continue;
             double ba, bb;
             if (!stencil_beta(la, va, nba, k - loa, step, npts, de, &ba)) continue;
@@ -854,12 +840,12 @@ __device__ int join_bin(const State &s, const double *mean, int w, int prev, dou
                 bk = k;
             }
         }
-        warp_argmin(best, bk);
+        block_argmin(best, bk);
         if (best < INFINITY) return bk;
     }
     double bd = INFINITY;
     int bk = 0x7fffffff;
-    for (int k = max(lob, prev + 1) + lane; k <= hia; k += 32) {
+    for (int k = max(lob, prev + 1) + first; k <= hia; k += by) {
         if (!va[k - loa] || !vb[k - lob]) continue;
         const double d = fabs((double)(2 * k - (lob + hia)));
         if (d < bd || (d == bd && k < bk)) {
@@ -867,20 +853,22 @@ __device__ int join_bin(const State &s, const double *mean, int w, int prev, dou
             bk = k;
         }
     }
-    warp_argmin(bd, bk);
+    block_argmin(bd, bk);
     return bd < INFINITY ? bk : -1;
 }
 
-// Joining is two launches over n sets of window means (set r at mean + r h W): k_join_bins, one warp per
+// Joining is two launches over n sets of window means (set r at mean + r h W): k_join_bins, one CTA per
 // pair and set, finds each pair's best join bin as if the pair were alone; k_stitch, one CTA per set,
 // searches a pair again, in order, where that bin does not lie behind the join before it (rare),
 // which gives the same bins as joining pair by pair, adds the shifts up in order, and gives every
 // bin its value from the last window joined at or below it.
-// Bound by float64 (2 FMA per cycle and SM) and latency, so the pairs are spread over the SMs and
-// the norm takes no exponential that cannot reach its last bit.  Ising L=64, 32 windows, with the
-// copies to the host: 230 us with one CTA going from pair to pair, 142 us; the jackknife's 16
-// resamples 3000 us one after the other, 184 us at once.
-__global__ void __launch_bounds__(32) k_join_bins(State s, const double *mean_all, double de, int step, int *joins_all,
+// Bound by float64 (2 FMA per cycle and SM) and latency, so the pairs are spread over the SMs, four
+// warps each (one: 30 us, four: 12; a pair searched again 12 us by one warp, 1 by all), the norm
+// takes no exponential that cannot reach its last bit, and its logarithm is one thread's.  Ising L=64,
+// 32 windows, with the copies to the host: 230 us with one CTA going from pair to pair, 96 us; the
+// jackknife's 16 resamples 3000 us one after the other, 133 us at once.
+constexpr int JOIN_THREADS = 128;
+__global__ void __launch_bounds__(JOIN_THREADS) k_join_bins(State s, const double *mean_all, double de, int step, int *joins_all,
                                                   double *at_all)
 {
     const int w = blockIdx.x, r = blockIdx.y;
@@ -920,16 +908,14 @@ __global__ void __launch_bounds__(1024) k_stitch(State s, const double *mean_all
         const int w = redo;
         __syncthreads();
         if (w + 1 >= h) break;
-        if (threadIdx.x < 32) {
-            const int kj = join_bin(s, mean, w, w > 0 ? joins[w - 1] : -1, de, step);
-            if (threadIdx.x == 0) {
-                joins[w] = kj;
-                if (kj < 0) {
-                    fail_s = 1;
-                } else {
-                    at[2 * w] = mean[(size_t)w * W + (kj - s.lo[w])];
-                    at[2 * w + 1] = mean[(size_t)(w + 1) * W + (kj - s.lo[w + 1])];
-                }
+        const int kj = join_bin(s, mean, w, w > 0 ? joins[w - 1] : -1, de, step);
+        if (threadIdx.x == 0) {
+            joins[w] = kj;
+            if (kj < 0) {
+                fail_s = 1;
+            } else {
+                at[2 * w] = mean[(size_t)w * W + (kj - s.lo[w])];
+                at[2 * w + 1] = mean[(size_t)(w + 1) * W + (kj - s.lo[w + 1])];
             }
         }
         __syncthreads();
@@ -979,7 +965,9 @@ __global__ void __launch_bounds__(1024) k_stitch(State s, const double *mean_all
         for (int b = threadIdx.x; b <= B; b += blockDim.x) // e^-80 of the largest term: no bit of the sum
             if (out[b] - mx > -80.0) sum += exp(out[b] - mx);
         sum = block_reduce_sum(sum);
-        const double cst = (mx + log(sum)) - target;
+        if (threadIdx.x == 0) sh_s = (mx + log(sum)) - target; // by one thread: 1024 logarithms take 5 us
+        __syncthreads();
+        const double cst = sh_s;
         for (int b = threadIdx.x; b <= B; b += blockDim.x)
             if (out[b] > -INFINITY) out[b] -= cst;
     } else {
@@ -1003,7 +991,7 @@ __global__ void __launch_bounds__(1024) k_stitch(State s, const double *mean_all
 cudaError_t launch_stitch(const State &s, int n, const double *mean, double de, int step, int norm,
                           double target, double *out, int *joins, double *at, int *ok, int B, cudaStream_t st)
 {
-    if (s.h > 1) k_join_bins<<<dim3(s.h - 1, n), 32, 0, st>>>(s, mean, de, step, joins, at);
+    if (s.h > 1) k_join_bins<<<dim3(s.h - 1, n), JOIN_THREADS, 0, st>>>(s, mean, de, step, joins, at);
     k_stitch<<<n, 1024, 0, st>>>(s, mean, de, step, norm, target, out, joins, at, ok, B);
     return cudaGetLastError();
 }
@@ -1113,7 +1101,7 @@ namespace rewl {
 // its own rounding error); only those, a tenth of the bins, take a quotient, an exponential and the
 // sums in float64.  Every bin does where float32 is too coarse to tell (large E/T), or where one bin holds
 // all the weight and c is made of the rest.  Ising L=64, 500
-// temperatures: 393 us with a float64 quotient per bin in three passes and two exponentials, 52 us.
+// temperatures: 393 us with a float64 quotient per bin in three passes and two exponentials, 51 us.
 // ---------------------------------------------------------------------------------------
 constexpr int THERMO_THREADS = 256;
 constexpr int THERMO_KEEP = 8; // weights a thread keeps between the two sums
@@ -1125,7 +1113,11 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     __shared__ double keep[THERMO_KEEP * THERMO_THREADS];
     __shared__ float mx_s[32], big_s[32];
     __shared__ int arg_s[32];
-    const double T = Ts[blockIdx.x], inv = 1.0 / T;
+    __shared__ double one_s; // float64 quotients are taken by one thread
+    const double T = Ts[blockIdx.x];
+    if (threadIdx.x == 0) one_s = 1.0 / T;
+    __syncthreads();
+    const double inv = one_s;
     const float invf = (float)inv;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     auto energy = [&](int b) { return model == 0 ? 4 * b - 2 * N : b - 2 * N; };
@@ -1200,7 +1192,9 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
             }
         s0 = block_reduce_sum(s0);
         s1 = block_reduce_sum(s1);
-        e1 = s1 / s0;
+        if (threadIdx.x == 0) one_s = s1 / s0;
+        __syncthreads();
+        e1 = one_s;
         s2 = 0.0;
         n = 0;
         for (int b = threadIdx.x; b <= B; b += blockDim.x)
@@ -1285,7 +1279,7 @@ __global__ void k_jack(const double *theta, int m, int B, double *err)
 
 cudaError_t launch_jack(const double *theta, int m, int B, double *err, cudaStream_t st)
 {
-    k_jack<<<(B + 256) / 256, 256, 0, st>>>(theta, m, B, err);
+    k_jack<<<(B + 64) / 64, 64, 0, st>>>(theta, m, B, err);
     return cudaGetLastError();
 }
 
