@@ -331,6 +331,11 @@ __device__ __forceinline__ void draw_block(const State &s, const MoveCfg &c, con
 
 // Words in shared memory that two warps of a CTA hand work over with.  (A fence after a plain load
 // would do the same, but holds the walker up for hundreds of cycles.)
+// Every lane loads such a word itself, so that what it reads or writes afterwards comes after its own
+// acquire, and the lanes then go on with the smallest value any of them saw (`agreed`): lanes of a warp
+// need not load at the same instant, and a branch on different values would part them before the
+// next full-mask vote.  A word is published by lane 0 after a __syncwarp, with release, so that it covers
+// what all lanes did.
 __device__ __forceinline__ int load_acquire(const int *p)
 {
     int v;
@@ -354,6 +359,8 @@ __device__ __forceinline__ void store_relaxed(int *p, int v)
     asm volatile("st.relaxed.cta.shared.b32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(p)), "r"(v) : "memory");
 }
 
+__device__ __forceinline__ int agreed(int v) { return (int)__reduce_min_sync(FULL, (unsigned)v); } // v >= 0
+
 // Polls of shared memory before a warp gives up on its partner: the first warp on the second, which
 // is never long, and the second, asleep between polls, on the first, which may rebuild float64
 // values for seconds (a tie in every addition of a bin's 10^8 visits).
@@ -371,8 +378,8 @@ __device__ __forceinline__ void draw_walker(const State &s, const MoveCfg &c, co
     __syncwarp();
     Drawn before;
     for (int g = 0; g < c.T + 64; g += 32) { // the first warp asks for 33 steps beyond the last
-        for (int it = 0; g + 32 - load_acquire(mem.ctl + 1) > MOVE_RING; ++it) {
-            if (load_acquire(mem.ctl + 2) || it > SLEEP_LIMIT) return;
+        for (int it = 0; g + 32 - agreed(load_acquire(mem.ctl + 1)) > MOVE_RING; ++it) {
+            if (__any_sync(FULL, load_acquire(mem.ctl + 2) != 0) || it > SLEEP_LIMIT) return;
             __nanosleep(50);
         }
         draw_block<ISING, false>(s, c, mem, slot, st0, g, before, lane);
@@ -541,13 +548,13 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
     cache_load(kstart);
     int table_age = table_life + 1; // visits since the table was taken
 
-    int g = 0; // steps drawn (as far as this warp knows)
+    int g = 0; // steps drawn (as far as this warp knows), the same in every lane
     Drawn before;
     // steps up to `upto` drawn; false if the partner warp does not come
     auto drawn = [&](int upto) -> bool {
         if (AHEAD) {
-            for (int it = 0; g < upto && it < SPIN_LIMIT; ++it) g = load_acquire(mem.ctl);
-            return __all_sync(FULL, g >= upto);
+            for (int it = 0; g < upto && it < SPIN_LIMIT; ++it) g = agreed(load_acquire(mem.ctl));
+            return g >= upto;
         }
         while (g < upto) {
             draw_block<ISING, REPLAY>(s, c, mem, slot, st0, g, before, lane);
@@ -865,14 +872,17 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
         }
         cache_age += stop;
         t += stop;
-        if (AHEAD) poll(mem.ctl, g, g < t + 33);
-        pe = mem.ring[(t + lane) & (MOVE_RING - 1)];
+        if (AHEAD) {
+            poll(mem.ctl, g, g < t + 33);
+            g = agreed(g);
+        }
+        pe = mem.ring[(t + lane) & (MOVE_RING - 1)]; // where g < t + 33 perhaps not written yet: read again below
         pnear = mem.near[(t + lane) & (MOVE_RING - 1)];
-        if (AHEAD && lane == 0) store_relaxed(mem.ctl + 1, t);
         nacc += mine && accj ? 1u : 0u;
         const int xlast = __shfl_sync(FULL, xa, stop - 1);
         x = stop > 0 ? xlast : x;
         __syncwarp();
+        if (AHEAD && lane == 0) store_release(mem.ctl + 1, t);
 
         if (__builtin_expect(open || stop == 0 || t >= T || g < t + 33, 0)) {
             if (!open && stop == 0) { // no step done and none to decide: cannot happen (lane 0 is never cut)
