@@ -463,8 +463,8 @@ __device__ __forceinline__ void move_walker_n(const State &s, const MoveCfg &c, 
         const unsigned bits = __ballot_sync(FULL, b < nb && (gmask == nullptr || gmask[b]));
         if (lane == 0) vis[i] = bits;
     }
-    __syncwarp();
     if (lane == 0) vis[(kstart - lo) >> 5] |= 1u << ((kstart - lo) & 31); // the start bin
+    __syncwarp(); // the first cache_load reads these words
     // the shadow of a running window ends the launch below (max |ln g| + T ln f) 2^32 < 2^62,
     // and ln f 2^32 must not round to zero; a frozen window adds nothing to it
     const bool lnf_ok = frozen || (lnf >= 0x1p-32 && lnf < 0x1p20 && mx + (double)T * lnf < 0x1p30);

@@ -33,3 +33,22 @@ def test_launch_lengths_around_block_and_ring(model, L, lnf):
         o.run(6)
         _same(g.state(), o.state(), FIELDS)
         g.close()
+
+
+# The start bin counts as visited from the first batch on: a launch that saw it as not visited would send
+# the steps from and to it to the float64 path.  The path taken, not only its result, is a function of the
+# state, so every repetition of a run counts the same number of float64 decisions.
+@pytest.mark.parametrize("model,L", [(0, 16), (10, 16)])
+def test_start_bin_is_visited_in_every_launch(model, L):
+    import paper_1402_2328_gb300.rewl as R
+    counts = []
+    for _ in range(4):
+        r = R.REWL(model, L, 4, 0.75, 8, 1e-9, 0.8, seed=I.seed_for(12, L), interval=200)
+        r.init()
+        r.run(max_rounds=50)
+        r.set_state("mask", np.zeros((r.h, r.W), np.uint8))  # only the start bin of each launch
+        r.set_state("lnf", np.full(4, 2.0 ** -16))
+        r.run(max_rounds=1)
+        counts.append(int(r.get_state("n_exact")[0]))
+        r.close()
+    assert len(set(counts)) == 1, counts
