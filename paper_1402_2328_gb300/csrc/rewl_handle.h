@@ -36,7 +36,7 @@ struct rewl_s {
     double *d_mean = nullptr, *d_out = nullptr;
     double *d_at = nullptr;
     int *d_joins = nullptr, *d_ok = nullptr;
-    void *d_jack = nullptr; // workspace of rewl_jackknife, made by its first call
+    void *d_jack = nullptr; // workspace of rewl_jackknife, at most 16 MB, made by its first call
     int8_t *d_spins = nullptr; // lattices in slot order for rewl_get_state, made by its first call
     rewl::DevStatus *h_status = nullptr; // pinned
     // graphs

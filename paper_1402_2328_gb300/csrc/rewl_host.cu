@@ -657,6 +657,11 @@ int rewl_abort(rewl_t r)
     return REWL_OK;
 }
 
+// Largest workspace that rewl_jackknife keeps: the 16 resamples of Ising L=64 32 x 16 take 2.6 MB of it, those of
+// Potts q=10 L=80 64 x 16 8 MB; where all of them take more, they are joined in several passes, each of
+// enough sets to fill the chip.
+constexpr size_t JACK_WORKSPACE = 16u << 20;
+
 int rewl_jackknife(rewl_t r, double *err, int cap, int norm)
 {
     if (!r || !err || (norm != 0 && norm != 1)) return REWL_ERR_INVALID_ARG;
@@ -670,26 +675,54 @@ int rewl_jackknife(rewl_t r, double *err, int cap, int norm)
     const double de = r->model == 0 ? 4.0 : 1.0;
     const int step = (r->model != 0 && r->q == 2) ? 2 : 1;
     const double target = norm == 0 ? (double)r->N * std::log((double)r->q) : std::log((double)r->q);
-    // workspace: the m resamples' values at their joins (16-byte aligned), window means and joined ln g, the
-    // error, joins and flags
+    // Joined `sets` resamples at once: their values at the joins (16-byte aligned), window means, joins and
+    // flags; behind them, where it fits too, every resample's joined ln g and the error.  Where one set is
+    // all there is room for, the buffers of rewl_stitch serve.
     const size_t m = (size_t)r->m, h = (size_t)r->h, W = (size_t)r->W, nb = (size_t)r->B + 1;
-    const size_t doubles = 2 * m * h + m * h * W + m * nb + nb, ints = m * h + m;
+    const size_t per = (2 * h + h * W) * 8 + (h + 1) * 4, result = (m + 1) * nb * 8;
+    bool inside = result + per <= JACK_WORKSPACE;
+    size_t sets = std::min(m, std::max<size_t>(1, (JACK_WORKSPACE - (inside ? result : 0)) / per));
     cudaError_t e = cudaSuccess;
-    if (!r->d_jack) e = cudaMalloc(&r->d_jack, doubles * 8 + ints * 4);
-    if (e != cudaSuccess) {
+    if (!inside && sets == 1) {
+        sets = 0;
+    } else if (!r->d_jack && cudaMalloc(&r->d_jack, sets * per + (inside ? result : 0)) != cudaSuccess) {
+        cudaGetLastError();
         r->d_jack = nullptr;
-        return r->cuda_fail(e, "rewl_jackknife");
+        inside = false;
+        sets = 0;
     }
-    double *at = (double *)r->d_jack, *means = at + 2 * m * h, *theta = means + m * h * W, *d_err = theta + m * nb;
-    int *joins = (int *)(d_err + nb), *d_oks = joins + m * h;
+    double *at = r->d_at, *means = r->d_mean, *theta = nullptr;
+    int *joins = r->d_joins, *d_oks = r->d_ok;
+    if (sets) {
+        at = (double *)r->d_jack;
+        means = at + 2 * sets * h;
+        double *end = means + sets * h * W;
+        if (inside) {
+            theta = end;
+            end += (m + 1) * nb;
+        }
+        joins = (int *)end;
+        d_oks = joins + sets * h;
+    } else {
+        sets = 1;
+    }
+    if (!inside) e = cudaMalloc(&theta, result);
+    if (e != cudaSuccess) return r->cuda_fail(e, "rewl_jackknife");
+    double *d_err = theta + m * nb;
     std::vector<int> oks(m, 0);
-    e = launch_loo_mean(r->st, means, r->stream);
-    if (e == cudaSuccess)
-        e = launch_stitch(r->st, r->m, means, de, step, norm, target, theta, joins, at, d_oks, r->B, r->stream);
+    for (size_t j = 0; j < m && e == cudaSuccess; j += sets) {
+        const int n = (int)std::min(sets, m - j);
+        e = launch_loo_mean(r->st, (int)j, n, means, r->stream);
+        if (e == cudaSuccess)
+            e = launch_stitch(r->st, n, means, de, step, norm, target, theta + j * nb, joins, at, d_oks, r->B,
+                              r->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(oks.data() + j, d_oks, n * sizeof(int), cudaMemcpyDeviceToHost, r->stream);
+    }
     if (e == cudaSuccess) e = launch_jack(theta, r->m, r->B, d_err, r->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(oks.data(), d_oks, m * sizeof(int), cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(err, d_err, nb * 8, cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
+    if (!inside) cudaFree(theta);
     if (e != cudaSuccess) return r->cuda_fail(e, "rewl_jackknife");
     for (int ok : oks)
         if (!ok) return r->fail(REWL_ERR_NOT_CONVERGED, "rewl_jackknife: a resample cannot be joined");

@@ -1226,11 +1226,11 @@ cudaError_t launch_thermo(const double *lng, int model, int L, const double *T, 
 
 namespace rewl {
 
-// Window means of the saved fragments leaving walker j out (walker order), [m][h][W].
-__global__ void k_loo_mean(State s, double *out_all)
+// Window means of the saved fragments leaving walker j0 + blockIdx.y out (walker order), [n][h][W].
+__global__ void k_loo_mean(State s, int j0, double *out_all)
 {
-    const int w = blockIdx.x, j = blockIdx.y, nb = s.hi[w] - s.lo[w] + 1;
-    double *out = out_all + (size_t)j * s.h * s.W;
+    const int w = blockIdx.x, j = j0 + blockIdx.y, nb = s.hi[w] - s.lo[w] + 1;
+    double *out = out_all + (size_t)blockIdx.y * s.h * s.W;
     for (int b = threadIdx.x; b < s.W; b += blockDim.x) {
         double v = 0.0;
         if (b < nb) {
@@ -1246,9 +1246,9 @@ __global__ void k_loo_mean(State s, double *out_all)
     }
 }
 
-cudaError_t launch_loo_mean(const State &s, double *out, cudaStream_t st)
+cudaError_t launch_loo_mean(const State &s, int j0, int n, double *out, cudaStream_t st)
 {
-    k_loo_mean<<<dim3(s.h, s.m), 256, 0, st>>>(s, out);
+    k_loo_mean<<<dim3(s.h, n), 256, 0, st>>>(s, j0, out);
     return cudaGetLastError();
 }
 

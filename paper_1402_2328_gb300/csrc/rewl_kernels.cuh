@@ -149,7 +149,8 @@ cudaError_t launch_bnd_decide(const State &s, int side, const double *half, cons
                               uint8_t *acc, int8_t *lat_out, cudaStream_t st);
 cudaError_t launch_bnd_import(const State &s, int side, const int *pbins, const uint8_t *acc,
                               const int8_t *plat, cudaStream_t st);
-cudaError_t launch_loo_mean(const State &s, double *out /*[m][h][W]*/, cudaStream_t st);
+// the n means that leave out walkers j0 .. j0+n-1
+cudaError_t launch_loo_mean(const State &s, int j0, int n, double *out /*[n][h][W]*/, cudaStream_t st);
 cudaError_t launch_jack(const double *theta /*[m][B+1]*/, int m, int B, double *err, cudaStream_t st);
 cudaError_t launch_thermo(const double *lng, int model, int L, const double *T, int nT, double *U,
                           double *C, cudaStream_t st);
