@@ -1,12 +1,79 @@
-"""The jackknife's many joins at once, in several passes over the resamples, against the oracle."""
+"""Joining where a pair's best bin is not the answer: bins out of order (the pair is searched again behind
+the join before it), overlaps with only a 3-point stencil or none, and the jackknife's many joins at
+once, in one pass over the resamples and in several, against the oracle.  Each case says what it is
+meant to reach, and an independent search checks that it does."""
 import numpy as np
 import pytest
 
 import oracle as O
-from tests.test_gpu_join import cuda_lib  # noqa: F401 (fixture)
+from tests.test_gpu_join import _planted, cuda_lib  # noqa: F401 (fixture)
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+
+def _beta(l, v, b, npts, step, de):
+    at = [b - step, b + step] + ([b - 2 * step, b + 2 * step] if npts == 5 else [])
+    if min(at) < 0 or max(at) >= len(l) or not all(v[i] for i in at):
+        return None
+    if npts == 5:
+        return ((8 * l[b + step] - l[b + 2 * step]) - 8 * l[b - step] + l[b - 2 * step]) / (12 * de * step)
+    return (l[b + step] - l[b - step]) / (2 * de * step)
+
+
+def _best_alone(model, lo, hi, mean, mask):
+    """Join bin of every pair as if it were alone, and the stencil that found it (5, 3, 0: none)."""
+    de, step = (4.0 if model == 0 else 1.0), (2 if model == 2 else 1)
+    bins, kinds = [], []
+    for w in range(len(lo) - 1):
+        win = [(mean[i][: hi[i] - lo[i] + 1], mask[i][: hi[i] - lo[i] + 1], lo[i]) for i in (w, w + 1)]
+        ks = [k for k in range(lo[w + 1], hi[w] + 1) if all(v[k - a] for _, v, a in win)]
+        for npts in (5, 3, 0):
+            if npts:
+                at = [(k, [_beta(l, v, k - a, npts, step, de) for l, v, a in win]) for k in ks]
+                c = [(abs(b[0] - b[1]), k) for k, b in at if None not in b]
+            else:
+                c = [(abs(2 * k - (lo[w + 1] + hi[w])), k) for k in ks]
+            if c:
+                bins.append(min(c)[1])
+                kinds.append(npts)
+                break
+    return bins, kinds
+
+
+def _out_of_order(bins):
+    return sum(b <= a for a, b in zip(bins, bins[1:]))
+
+
+# window i overlaps i + 1 in ten bins and no other window, so each pair's stencil is planted by itself:
+# visited runs of three bins leave only the 3-point one, single bins none
+@pytest.mark.parametrize("model,m", [(0, 1), (3, 2)])
+@pytest.mark.parametrize("norm", [0, 1])
+def test_stencils_of_each_pair(model, m, norm):
+    L = 17 if model == 0 else 12
+    B = O.num_bins(model, L)
+    lo = (21 * np.arange(B // 21 - 1)).astype(np.int32)
+    hi = lo + 30
+    hi[-1] = B
+    g, o = _planted(model, L, lo, hi, m, 77 + model, 0.3, 0.0)
+    mask = o.state()["mask"].copy()
+    want = [(5, 3, 0)[w % 3] for w in range(len(lo) - 1)]
+    for w, kind in enumerate(want):
+        for k in range(lo[w + 1], hi[w] + 1):
+            seen = kind == 5 or (kind == 3 and (k - lo[w + 1]) % 4 < 3) or (kind == 0 and (k - lo[w + 1]) % 2 == 0)
+            mask[w, k - lo[w]] = mask[w + 1, k - lo[w + 1]] = seen
+    g.set_state("mask", mask)
+    o.put_window(mask=mask)
+    mean = [o.window_mean(w) for w in range(len(lo))]
+    assert _best_alone(model, lo, hi, mean, mask)[1] == want
+    a, ja = g.stitch(norm)
+    b, jb = o.stitch(norm)
+    assert np.array_equal(ja, jb)
+    fin = np.isfinite(b)
+    assert np.array_equal(np.isfinite(a), fin)
+    # sums of exponentials in another order: a few last bits of values up to a few thousand
+    assert np.max(np.abs(a[fin] - b[fin])) < 1e-11
+    g.close()
 
 
 def _finished_pair(model, L, h, m, interval, seed, lnf_final=2.0 ** -3):
@@ -34,6 +101,23 @@ def _same_error(g, o, norm):
     tol = 4 * g.m ** 1.5 * 2.0 ** -53 * big
     assert np.max(np.abs(a[fin] - b[fin])) <= tol
     assert np.max(b[fin]) > 1e3 * tol  # and the error is something
+
+
+# pairs searched again in some resamples, fewer and more windows than are joined by one CTA alone; model 2
+# has stencils of step 2
+@pytest.mark.parametrize("model,L,h,m,interval,seed", [
+    (0, 8, 6, 3, 400, 1), (0, 12, 8, 5, 800, 7), (2, 8, 6, 3, 600, 9), (3, 8, 12, 2, 800, 6),
+    (0, 16, 12, 4, 1500, 4), (10, 10, 20, 3, 1500, 5), (0, 16, 40, 2, 2000, 8)])
+@pytest.mark.parametrize("norm", [0, 1])
+def test_jackknife_with_bins_out_of_order(model, L, h, m, interval, seed, norm):
+    g, o = _finished_pair(model, L, h, m, interval, seed)
+    s = o.state()
+    frag = s["frag"].reshape(h, m, -1)
+    again = [_out_of_order(_best_alone(model, o.lo, o.hi, (frag.sum(1) - frag[:, j]) / (m - 1), s["mask"])[0])
+             for j in range(m)]
+    assert max(again) > 0  # searched again in some resample
+    _same_error(g, o, norm)
+    g.close()
 
 
 # 1024 resamples take more than the workspace that a handle keeps: several passes, with the resamples'
