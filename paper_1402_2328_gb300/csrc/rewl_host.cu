@@ -74,17 +74,6 @@ int check_windows(int B, const std::vector<int> &lo, const std::vector<int> &hi)
 
 } // namespace
 
-// Makes the pages of a caller's output buffer present before the device writes to it.  A copy to pages
-// that do not exist yet (a large fresh allocation) takes a fault per page in the driver: 6.2 MB took
-// 4.8 ms, with the pages made here first 0.16 ms.
-static void touch_pages(void *p, size_t bytes)
-{
-    if (bytes < (1u << 18)) return;
-    volatile unsigned char *c = static_cast<volatile unsigned char *>(p);
-    for (size_t i = 0; i < bytes; i += 4096) c[i] = 0;
-    c[bytes - 1] = 0;
-}
-
 static int walkers_per_block(const rewl_t r)
 {
     const size_t per = move_smem_per_walker(r->N, r->W);
@@ -1014,7 +1003,6 @@ int rewl_get_state(rewl_t r, const char *name, void *out, size_t bytes)
                 std::memcpy((int8_t *)out + i * N, all.data() + (size_t)cfg[i] * r->st.spin_stride, N);
             return REWL_OK;
         }
-        touch_pages(out, bytes);
         e = launch_gather_spins(r->st, r->d_spins, r->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, r->d_spins, bytes, cudaMemcpyDeviceToHost, r->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
@@ -1025,7 +1013,6 @@ int rewl_get_state(rewl_t r, const char *name, void *out, size_t bytes)
         const size_t nbytes = (size_t)r->h * r->W * 8;
         if (bytes != nbytes) return r->fail(REWL_ERR_BUFFER_TOO_SMALL, "lng_mean: bytes mismatch");
         e = launch_window_mean(r->st, r->d_mean, r->stream);
-        touch_pages(out, nbytes);
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, r->d_mean, nbytes, cudaMemcpyDeviceToHost, r->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
         if (e != cudaSuccess) return r->cuda_fail(e, "lng_mean");
@@ -1043,7 +1030,6 @@ int rewl_get_state(rewl_t r, const char *name, void *out, size_t bytes)
     Field fd;
     if (!field(r, f, fd)) return r->fail(REWL_ERR_INVALID_ARG, "unknown field " + f);
     if (bytes != fd.bytes) return r->fail(REWL_ERR_BUFFER_TOO_SMALL, f + ": bytes mismatch");
-    touch_pages(out, bytes);
     e = cudaMemcpyAsync(out, fd.dev, bytes, cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
     if (e != cudaSuccess) return r->cuda_fail(e, "rewl_get_state");

@@ -133,6 +133,16 @@ def _ptr(a):
     return a.ctypes.data_as(C.c_void_p)
 
 
+def _present(a):
+    """The array, freshly made, with its pages present.  A large one has none yet, and a device-to-host copy
+    takes a fault per page in the driver: 6.2 MB took 4.8 ms, with the pages made here first 0.16 ms."""
+    if a.nbytes >= 1 << 18:
+        b = a.reshape(-1).view(np.uint8)
+        b[::4096] = 0
+        b[-1] = 0
+    return a
+
+
 def _stream_ptr(stream):
     if stream is None:
         try:
@@ -327,7 +337,7 @@ class REWL:
 
     def get_state(self, field: str) -> np.ndarray:
         dt, code = _FIELDS[field]
-        out = np.zeros(self._shape(code), dt)
+        out = _present(np.zeros(self._shape(code), dt))
         _check(self._lib.rewl_get_state(self._h, field.encode(), _ptr(out), out.nbytes), self._h)
         return out
 
