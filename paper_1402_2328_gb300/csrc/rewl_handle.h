@@ -37,7 +37,8 @@ struct rewl_s {
     double *d_at = nullptr;
     int *d_joins = nullptr, *d_ok = nullptr;
     void *d_jack = nullptr; // workspace of rewl_jackknife, at most 16 MB, made by its first call
-    int8_t *d_spins = nullptr; // lattices in slot order for rewl_get_state, made by its first call
+    int8_t *d_stage = nullptr; // [stage_slots][N] lattices in slot order, for rewl_get_state
+    int stage_slots = 0;
     rewl::DevStatus *h_status = nullptr; // pinned
     // graphs
     cudaGraphExec_t graph = nullptr;

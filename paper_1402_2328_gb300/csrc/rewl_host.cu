@@ -108,7 +108,7 @@ static void release(rewl_t r)
     void *ptrs[] = {s.spins, s.cfg, s.k, s.lng, s.H, s.step, s.acc, s.pstep, s.restarts, s.flat,
                     r->d_lohi, s.lnf, s.iter, s.finished, s.mask, s.swap_att, s.swap_acc,
                     s.it1_round, s.mode, s.frag, s.hem, s.status, s.sync, r->d_mean, r->d_out, r->d_joins,
-                    r->d_ok, r->d_at, r->d_jack, r->d_spins};
+                    r->d_ok, r->d_at, r->d_jack, r->d_stage};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (r->h_status) cudaFreeHost(r->h_status);
@@ -119,9 +119,13 @@ static void release(rewl_t r)
     r->d_joins = r->d_ok = nullptr;
     r->d_at = nullptr;
     r->d_jack = nullptr;
-    r->d_spins = nullptr;
+    r->d_stage = nullptr;
     r->allocated = false;
 }
+
+// Lattices in slot order on their way to the host (rewl_get_state): 8 MB hold those of Potts L=80 64 x 16 at
+// once; more take several copies.
+constexpr size_t STAGE_BYTES = 8u << 20;
 
 static int allocate(rewl_t r)
 {
@@ -176,6 +180,8 @@ static int allocate(rewl_t r)
     r->d_joins = dmalloc<int>(h, e);
     r->d_at = dmalloc<double>(2 * h, e);
     r->d_ok = dmalloc<int>(1, e);
+    r->stage_slots = (int)std::min(nw, std::max<size_t>(1, STAGE_BYTES / (size_t)r->N));
+    r->d_stage = dmalloc<int8_t>((size_t)r->stage_slots * r->N, e);
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&r->h_status, sizeof(DevStatus), cudaHostAllocDefault);
     if (e != cudaSuccess) {
         release(r);
@@ -989,22 +995,12 @@ int rewl_get_state(rewl_t r, const char *name, void *out, size_t bytes)
     if (f == "spins") { // gather per slot through the slot -> configuration map
         const size_t N = (size_t)r->N, nw = (size_t)r->nw;
         if (bytes != nw * N) return r->fail(REWL_ERR_BUFFER_TOO_SMALL, "spins: bytes mismatch");
-        if (!r->d_spins && cudaMalloc((void **)&r->d_spins, nw * N) != cudaSuccess) {
-            cudaGetLastError(); // no device memory for the ordered copy: order it on the host
-            r->d_spins = nullptr;
-            std::vector<int> cfg(nw);
-            std::vector<int8_t> all(nw * (size_t)r->st.spin_stride);
-            e = cudaMemcpyAsync(cfg.data(), r->st.cfg, nw * 4, cudaMemcpyDeviceToHost, r->stream);
+        for (size_t i = 0; i < nw && e == cudaSuccess; i += (size_t)r->stage_slots) {
+            const size_t n = std::min((size_t)r->stage_slots, nw - i);
+            e = launch_gather_spins(r->st, (int)i, (int)n, r->d_stage, r->stream);
             if (e == cudaSuccess)
-                e = cudaMemcpyAsync(all.data(), r->st.spins, all.size(), cudaMemcpyDeviceToHost, r->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
-            if (e != cudaSuccess) return r->cuda_fail(e, "get spins");
-            for (size_t i = 0; i < nw; ++i)
-                std::memcpy((int8_t *)out + i * N, all.data() + (size_t)cfg[i] * r->st.spin_stride, N);
-            return REWL_OK;
+                e = cudaMemcpyAsync((int8_t *)out + i * N, r->d_stage, n * N, cudaMemcpyDeviceToHost, r->stream);
         }
-        e = launch_gather_spins(r->st, r->d_spins, r->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(out, r->d_spins, bytes, cudaMemcpyDeviceToHost, r->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
         if (e != cudaSuccess) return r->cuda_fail(e, "get spins");
         return REWL_OK;

@@ -671,13 +671,10 @@ cudaError_t launch_set_done(const State &s, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------------------------------
-// Joining (Sec. 3, Eq. 2).
-// ---------------------------------------------------------------------------------------
-// Lattices in slot order, one CTA per slot.
-__global__ void k_gather_spins(State s, int8_t *out)
+// Lattices in slot order from slot `first` on, one CTA per slot.
+__global__ void k_gather_spins(State s, int first, int8_t *out)
 {
-    const int8_t *src = s.spins + (size_t)s.cfg[blockIdx.x] * s.spin_stride;
+    const int8_t *src = s.spins + (size_t)s.cfg[first + (int)blockIdx.x] * s.spin_stride;
     int8_t *dst = out + (size_t)blockIdx.x * s.N;
     if (s.vec_spins) { // N a multiple of 16
         for (int i = threadIdx.x; i < s.N >> 4; i += blockDim.x)
@@ -687,12 +684,15 @@ __global__ void k_gather_spins(State s, int8_t *out)
     }
 }
 
-cudaError_t launch_gather_spins(const State &s, int8_t *out, cudaStream_t st)
+cudaError_t launch_gather_spins(const State &s, int first, int n, int8_t *out, cudaStream_t st)
 {
-    k_gather_spins<<<s.nw, 128, 0, st>>>(s, out);
+    k_gather_spins<<<n, 128, 0, st>>>(s, first, out);
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------------------
+// Joining (Sec. 3, Eq. 2).
+// ---------------------------------------------------------------------------------------
 __global__ void k_window_mean(State s, double *out)
 {
     const int w = blockIdx.x, nb = s.hi[w] - s.lo[w] + 1;

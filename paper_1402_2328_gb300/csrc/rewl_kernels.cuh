@@ -133,7 +133,8 @@ cudaError_t launch_round_tail(const State &s, double flatness, double lnf_final,
 cudaError_t launch_set_done(const State &s, cudaStream_t st);
 // joint density of states g(E, M) (rewl_em.cu)
 cudaError_t launch_measure_em(const State &s, cudaStream_t st);
-cudaError_t launch_gather_spins(const State &s, int8_t *out /*[nw][N]*/, cudaStream_t st);
+// lattices of slots first .. first+n-1
+cudaError_t launch_gather_spins(const State &s, int first, int n, int8_t *out /*[n][N]*/, cudaStream_t st);
 cudaError_t launch_window_mean(const State &s, double *out /*[h][W]*/, cudaStream_t st);
 // n joins at once: of the window means at mean + r h W, r = 0 .. n-1
 cudaError_t launch_stitch(const State &s, int n, const double *mean, double de, int step, int norm,
