@@ -670,11 +670,11 @@ int rewl_jackknife(rewl_t r, double *err, int cap, int norm)
     const double de = r->model == 0 ? 4.0 : 1.0;
     const int step = (r->model != 0 && r->q == 2) ? 2 : 1;
     const double target = norm == 0 ? (double)r->N * std::log((double)r->q) : std::log((double)r->q);
-    // Joined `sets` resamples at once: their values at the joins (16-byte aligned), window means, joins and
-    // flags; behind them, where it fits too, every resample's joined ln g and the error.  Where one set is
-    // all there is room for, the buffers of rewl_stitch serve.
+    // Joined `sets` resamples at once: their values at the joins (16-byte aligned), window means and joins;
+    // behind the means, where it fits too, every resample's joined ln g, the error and every resample's flag.
+    // Where one set is all there is room for, the buffers of rewl_stitch serve.
     const size_t m = (size_t)r->m, h = (size_t)r->h, W = (size_t)r->W, nb = (size_t)r->B + 1;
-    const size_t per = (2 * h + h * W) * 8 + (h + 1) * 4, result = (m + 1) * nb * 8;
+    const size_t per = (2 * h + h * W) * 8 + h * 4, result = (m + 1) * nb * 8 + ((m + 1) / 2) * 8;
     bool inside = result + per <= JACK_WORKSPACE;
     size_t sets = std::min(m, std::max<size_t>(1, (JACK_WORKSPACE - (inside ? result : 0)) / per));
     cudaError_t e = cudaSuccess;
@@ -687,34 +687,33 @@ int rewl_jackknife(rewl_t r, double *err, int cap, int norm)
         sets = 0;
     }
     double *at = r->d_at, *means = r->d_mean, *theta = nullptr;
-    int *joins = r->d_joins, *d_oks = r->d_ok;
+    int *joins = r->d_joins;
     if (sets) {
         at = (double *)r->d_jack;
         means = at + 2 * sets * h;
         double *end = means + sets * h * W;
         if (inside) {
             theta = end;
-            end += (m + 1) * nb;
+            end += result / 8;
         }
         joins = (int *)end;
-        d_oks = joins + sets * h;
     } else {
         sets = 1;
     }
     if (!inside) e = cudaMalloc(&theta, result);
     if (e != cudaSuccess) return r->cuda_fail(e, "rewl_jackknife");
     double *d_err = theta + m * nb;
+    int *d_oks = (int *)(d_err + nb);
     std::vector<int> oks(m, 0);
     for (size_t j = 0; j < m && e == cudaSuccess; j += sets) {
         const int n = (int)std::min(sets, m - j);
         e = launch_loo_mean(r->st, (int)j, n, means, r->stream);
         if (e == cudaSuccess)
-            e = launch_stitch(r->st, n, means, de, step, norm, target, theta + j * nb, joins, at, d_oks, r->B,
+            e = launch_stitch(r->st, n, means, de, step, norm, target, theta + j * nb, joins, at, d_oks + j, r->B,
                               r->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(oks.data() + j, d_oks, n * sizeof(int), cudaMemcpyDeviceToHost, r->stream);
     }
     if (e == cudaSuccess) e = launch_jack(theta, r->m, r->B, d_err, r->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(oks.data(), d_oks, m * sizeof(int), cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(err, d_err, nb * 8, cudaMemcpyDeviceToHost, r->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
     if (!inside) cudaFree(theta);
