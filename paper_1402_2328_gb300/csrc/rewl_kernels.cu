@@ -857,17 +857,24 @@ __device__ int join_bin(const State &s, const double *mean, int w, int prev, dou
     return bd < INFINITY ? bk : -1;
 }
 
-// Joining is two launches over n sets of window means (set r at mean + r h W): k_join_bins, one CTA per
-// pair and set, finds each pair's best join bin as if the pair were alone; k_stitch, one CTA per set,
-// searches a pair again, in order, where that bin does not lie behind the join before it (rare),
-// which gives the same bins as joining pair by pair, adds the shifts up in order, and gives every
-// bin its value from the last window joined at or below it.
+// Joining n sets of window means (set r at mean + r h W): k_join_bins, one CTA per pair and set, finds each
+// pair's best join bin as if the pair were alone; k_stitch, one CTA per set, searches a pair again, in
+// order, where that bin does not lie behind the join before it, which gives the same bins as joining pair
+// by pair, adds the shifts up in order, and gives every bin its value from the last window joined at or
+// below it.
 // Bound by float64 (2 FMA per cycle and SM) and latency, so the pairs are spread over the SMs, four
-// warps each (one: 30 us, four: 12; a pair searched again 12 us by one warp, 1 by all), the norm
-// takes no exponential that cannot reach its last bit, and its logarithm is one thread's.  Ising L=64,
-// 32 windows, with the copies to the host: 230 us with one CTA going from pair to pair, 96 us; the
-// jackknife's 16 resamples 3000 us one after the other, 133 us at once.
-constexpr int JOIN_THREADS = 128;
+// warps each (one: 30 us, four: 12), the norm takes no exponential that cannot reach its last bit, and its
+// logarithm is one thread's.  Ising L=64, 32 windows, with the copies to the host: 212 us with one CTA going
+// from pair to pair, 91 us; the jackknife's 16 resamples 3000 us one after the other, 131 us at once.
+// k_stitch has 256 threads: with 1024 of 64 registers each, a search again and the passes over all bins
+// took longer (Ising L=16 8 x 8 89 us, now 74; Potts L=40 64 x 4 138, now 115).
+// A few small windows are searched by k_stitch alone (join_alone): the launch of k_join_bins and the searches
+// again, which noisy windows need more of, cost as much as they save.  us, alone / by k_join_bins: Ising L=8
+// 2 x 4 50 / 53, Ising L=16 4 x 32 62 / 65, 8 x 8 75 / 78, but 78 / 65 with 8 windows of 292 bins and
+// 163 / 76 with 32 of 118.
+constexpr int JOIN_THREADS = 128, STITCH_THREADS = 256;
+__host__ __device__ inline bool join_alone(const State &s) { return s.h <= 2 || (s.h <= 8 && s.W <= 192); }
+
 __global__ void __launch_bounds__(JOIN_THREADS) k_join_bins(State s, const double *mean_all, double de, int step, int *joins_all,
                                                   double *at_all)
 {
@@ -882,11 +889,11 @@ __global__ void __launch_bounds__(JOIN_THREADS) k_join_bins(State s, const doubl
     }
 }
 
-// out + r (B+1): joined ln g of set r; joins, at and ok: as k_join_bins left them, [n][h], [n][h][2], [n];
-// at becomes the windows' shifts.
-__global__ void __launch_bounds__(1024) k_stitch(State s, const double *mean_all, double de, int step, int norm,
-                                                 double target, double *out_all, int *joins_all, double *at_all,
-                                                 int *ok_all, int B)
+// out + r (B+1): joined ln g of set r; joins, at and ok: [n][h], [n][h][2], [n], the first two as k_join_bins left
+// them unless join_alone; at becomes the windows' shifts.
+__global__ void __launch_bounds__(STITCH_THREADS)
+    k_stitch(State s, const double *mean_all, double de, int step, int norm, double target, double *out_all,
+             int *joins_all, double *at_all, int *ok_all, int B)
 {
     const int W = s.W, h = s.h;
     const double *mean = mean_all + (size_t)blockIdx.x * h * W;
@@ -894,11 +901,14 @@ __global__ void __launch_bounds__(1024) k_stitch(State s, const double *mean_all
     int *joins = joins_all + (size_t)blockIdx.x * h, *ok = ok_all + blockIdx.x;
     __shared__ int redo, fail_s;
     __shared__ double sh_s;
-    __shared__ double2 step_s[1024];
+    __shared__ double2 step_s[STITCH_THREADS];
     if (threadIdx.x == 0) {
         fail_s = 0;
         sh_s = 0.0;
     }
+    if (join_alone(s)) // no pair has a join yet
+        for (int w = threadIdx.x; w + 1 < h; w += blockDim.x) joins[w] = -1;
+    __syncthreads();
     for (int w0 = 0;;) { // the first pair from w0 on whose join is not behind the one before
         if (threadIdx.x == 0) redo = h - 1;
         __syncthreads();
@@ -965,7 +975,7 @@ __global__ void __launch_bounds__(1024) k_stitch(State s, const double *mean_all
         for (int b = threadIdx.x; b <= B; b += blockDim.x) // e^-80 of the largest term: no bit of the sum
             if (out[b] - mx > -80.0) sum += exp(out[b] - mx);
         sum = block_reduce_sum(sum);
-        if (threadIdx.x == 0) sh_s = (mx + log(sum)) - target; // by one thread: 1024 logarithms take 5 us
+        if (threadIdx.x == 0) sh_s = (mx + log(sum)) - target; // by one thread: a logarithm of every thread takes 5 us
         __syncthreads();
         const double cst = sh_s;
         for (int b = threadIdx.x; b <= B; b += blockDim.x)
@@ -991,8 +1001,8 @@ __global__ void __launch_bounds__(1024) k_stitch(State s, const double *mean_all
 cudaError_t launch_stitch(const State &s, int n, const double *mean, double de, int step, int norm,
                           double target, double *out, int *joins, double *at, int *ok, int B, cudaStream_t st)
 {
-    if (s.h > 1) k_join_bins<<<dim3(s.h - 1, n), JOIN_THREADS, 0, st>>>(s, mean, de, step, joins, at);
-    k_stitch<<<n, 1024, 0, st>>>(s, mean, de, step, norm, target, out, joins, at, ok, B);
+    if (!join_alone(s)) k_join_bins<<<dim3(s.h - 1, n), JOIN_THREADS, 0, st>>>(s, mean, de, step, joins, at);
+    k_stitch<<<n, STITCH_THREADS, 0, st>>>(s, mean, de, step, norm, target, out, joins, at, ok, B);
     return cudaGetLastError();
 }
 

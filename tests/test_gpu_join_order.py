@@ -76,6 +76,25 @@ def test_stencils_of_each_pair(model, m, norm):
     g.close()
 
 
+# on both sides of the limits up to which one CTA searches all pairs: 2 windows whatever their size, 8
+# windows, 192 bins
+@pytest.mark.parametrize("h,W", [(2, 900), (8, 192), (8, 193), (9, 150)])
+def test_pairs_searched_by_one_cta_and_by_many(h, W):
+    model, L = 0, 32
+    B = O.num_bins(model, L)
+    lo = ((B - W + 1) * np.arange(h) // (h - 1)).astype(np.int32)
+    hi = (lo + W - 1).astype(np.int32)
+    g, o = _planted(model, L, lo, hi, 2, 90 + h + W, 3.0, 0.0)
+    assert (g.h, g.W) == (h, W)
+    a, ja = g.stitch()
+    b, jb = o.stitch()
+    assert np.array_equal(ja, jb)
+    assert np.array_equal(np.isfinite(a), np.isfinite(b))
+    fin = np.isfinite(b)
+    assert np.max(np.abs(a[fin] - b[fin])) < 1e-11  # as above
+    g.close()
+
+
 def _finished_pair(model, L, h, m, interval, seed, lnf_final=2.0 ** -3):
     """Short runs taken through all their iterations (every check counts as flat): noisy fragments."""
     import paper_1402_2328_gb300.rewl as R
