@@ -1180,7 +1180,10 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     // one bin holds nearly all the weight: the others do not reach `enough`, so every bin is taken at once
     // (either way is right; what this misses is found by s2 below)
     const bool frozen = mx - next > 43.0f - __logf((float)(B + 1) * (float)N * (float)N);
-    double s0, e1, s2;
+    // energies from the bin of the largest exponent, so that a mean next to it keeps all its digits: c of a
+    // frozen lattice is a sum over the other bins
+    auto rel = [&](int b) { return (double)(energy(b) - energy(arg)); };
+    double s0, e1, s2; // e1: relative mean
     for (bool all = frozen || !(slack < 8.0f && fabs(T) < INFINITY);; all = true) {
         auto exponent = [&](int b) {
             const double E = (double)energy(b);
@@ -1207,7 +1210,7 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
                 if (n < THERMO_KEEP) keep[n * THERMO_THREADS + threadIdx.x] = w;
                 ++n;
                 s0 += w;
-                s1 += w * energy(b);
+                s1 += w * rel(b);
             }
         s0 = block_reduce_sum(s0);
         s1 = block_reduce_sum(s1);
@@ -1220,14 +1223,14 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
             if (counts(b)) {
                 const double w = n < THERMO_KEEP ? keep[n * THERMO_THREADS + threadIdx.x] : exp(exponent(b) - ref);
                 ++n;
-                const double de = energy(b) - e1;
+                const double de = rel(b) - e1;
                 s2 += w * de * de;
             }
         s2 = block_reduce_sum(s2);
         if (all || s2 >= enough * s0) break; // else nearly one bin alone (low T): again with every bin
     }
     if (threadIdx.x == 0) {
-        U[blockIdx.x] = e1 / N;
+        U[blockIdx.x] = (energy(arg) + e1) / N;
         Cv[blockIdx.x] = s2 / s0 / ((double)N * T * T);
     }
 }
