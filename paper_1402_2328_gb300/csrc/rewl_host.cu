@@ -151,7 +151,7 @@ static int allocate(rewl_t r)
     s.spin_stride = (r->N + 15) & ~15;
     s.vec_spins = (r->N & 15) == 0;
     s.magic = (uint32_t)((0x100000000ULL + (uint64_t)r->L - 1) / (uint64_t)r->L);
-    if (!move_fits(r->N, r->W))
+    if (!move_fits(r->N, r->W) || move_smem_per_walker(r->N, r->W) > MAX_SMEM_PER_CTA)
         return r->fail(REWL_ERR_INVALID_ARG, "lattice and window do not fit in shared memory");
     s.spins = dmalloc<int8_t>(nw * s.spin_stride, e);
     s.cfg = dmalloc<int>(nw, e);

@@ -106,8 +106,9 @@ inline bool draw_ahead_pays(long long walkers, int sms, int walkers_per_cta, siz
     const long long fit = (long long)(MAX_SMEM_PER_CTA / smem_per_walker);
     return walkers_per_cta <= 8 && walkers <= sms * (fit < 8 ? fit : 8);
 }
-// The largest lattice and window accepted: 3 bytes per site and 8 per bin within one CTA, which
-// covers move_smem_per_walker for every size it admits.
+// The largest lattice and window accepted: 3 bytes per site and 8 per bin within one CTA.  It leaves the batch
+// scratch out, so it covers move_smem_per_walker only for rows no wider than a lattice has bins
+// (W <= 2N + 1, as in every handle); a replay's wider rows run one thread per walker (replay_layout).
 __host__ __device__ inline bool move_fits(int N, int W)
 {
     return (size_t)((N + 15) & ~15) + (size_t)((W + 3) & ~3) * 8u + (size_t)visw(W) * 4u +

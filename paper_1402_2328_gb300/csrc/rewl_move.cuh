@@ -107,13 +107,6 @@ __device__ __forceinline__ float ulpf(float x)
     return e > 23 ? __int_as_float((e - 23) << 23) : 0x1p-126f;
 }
 
-__device__ __forceinline__ float warp_maxf(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(FULL, v, o));
-    return v;
-}
-
 // visits of bin b since the launch started: the shadow grew by lnfq per visit
 __device__ __forceinline__ uint32_t visits(const long long *V, const double *glng, int b, long long lnfq)
 {
