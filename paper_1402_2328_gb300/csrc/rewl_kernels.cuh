@@ -72,8 +72,9 @@ constexpr int MOVE_TAB_BYTES = 9 * 80;
 constexpr int MOVE_RING = 128;
 constexpr int MOVE_SCRATCH_BYTES = MOVE_TAB_BYTES + 9 * 36 * 4 + 24 * 16 + 32 * 4 + MOVE_RING * 20 + 16;
 // Largest ln f at which a batch is walked through the ratio table.  Above it the visits of the batch
-// itself leave too many steps undecided (us per launch, Potts L=80 64 x 16 and Ising L=64 32 x 16,
-// table / running walk: 535 / 551 and 430 / 429 at 2^-6, 594 / 553 and 480 / 429 at 2^-5).
+// itself leave too many steps undecided (us per launch, table / running walk, at 1, 1.2, 1.49 and 2 times 2^-6:
+// Potts L=80 64 x 16 541 / 569, 558 / 572, 578 / 571, 606 / 573; Ising L=64 32 x 16 424 / 440, 436 / 440,
+// 453 / 443, 476 / 443; Ising L=32 8 x 8 425 / 497, 440 / 496, 456 / 496, 482 / 499).
 constexpr float TABLE_WALK_LNF = 0x1.8p-6f;
 // Largest ln f at which undecided steps are rare enough to be taken one by one: verifying the whole path
 // costs the walk registers (Potts L=40 at 2^-10: 490 us one by one, 474 verified, Ising L=64 at 2^-8 433
@@ -88,7 +89,10 @@ constexpr float SURE_DRIFT = 0x1p-6f, VERIFIED_DRIFT = 0x1p-5f;
 // changes the bin by 4 at most).
 constexpr int CACHE_LO = 6, CACHE_HI = 25;
 // Smallest lattices whose batches are 32 and 16 steps (smaller ones: 8).  Sites soon repeat on a
-// small lattice: a batch ends after about 5 steps on 64 sites, 13 on 256, 24 on 1024.
+// small lattice: a batch ends after about 5 steps on 64 sites, 13 on 256, 24 on 1024.  us per launch of Ising
+// 8 x 8 at ln f = 1 / 2^-9 / 2^-20: 32 steps against 16 on L=21 730 / 533 / 429 and 631 / 534 / 422, on
+// L=22 711 / 482 / 400 and 621 / 504 / 406, on L=28 586 / 363 / 291 and 575 / 442 / 356; 16 steps against 8 on
+// L=9 1193 / 943 / 833 and 1051 / 935 / 829, on L=10 1083 / 865 / 750 and 988 / 884 / 774.
 constexpr int BATCH32_SITES = 450, BATCH16_SITES = 100;
 
 // Shared memory of one walker in the move kernel: lattice and stamps (a byte each per site, padded
@@ -100,7 +104,9 @@ __host__ __device__ inline size_t move_smem_per_walker(int N, int W)
            (size_t)MOVE_SCRATCH_BYTES;
 }
 // Whether a second warp per walker pays: it takes the drawing off the walker's chain, as long as
-// all walkers of the launch are still resident at once (128 registers: 16 warps per SM).
+// all walkers of the launch are still resident at once (128 registers: 16 warps per SM).  us per launch, with
+// and without it, Ising L=64 at 2^-20: 512 walkers 253 / 373, 1216 (8 per SM) 328 / 423, 1280 476 / 466; at
+// ln f = 1 460 / 582, 590 / 665, 942 / 807; Potts L=20 at 2^-20 1216 walkers 633 / 771, 1280 936 / 876.
 inline bool draw_ahead_pays(long long walkers, int sms, int walkers_per_cta, size_t smem_per_walker)
 {
     const long long fit = (long long)(MAX_SMEM_PER_CTA / smem_per_walker);
