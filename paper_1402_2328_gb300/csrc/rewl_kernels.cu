@@ -1102,6 +1102,40 @@ cudaError_t launch_seqadd(const double *x, const double *f, const uint32_t *c, d
 
 namespace rewl {
 
+// Sums of a and b over the CTA, added in the order of block_reduce_sum: a becomes its sum, b the quotient of
+// theirs.  The caller has a barrier before the next call.
+__device__ __forceinline__ void block_mean(double &a, double &b)
+{
+    __shared__ double sa[32], sb[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(FULL, a, o);
+        b += __shfl_xor_sync(FULL, b, o);
+    }
+    if (lane == 0) {
+        sa[wid] = a;
+        sb[wid] = b;
+    }
+    __syncthreads();
+    if (wid == 0) {
+        a = lane < (int)(blockDim.x >> 5) ? sa[lane] : 0.0;
+        b = lane < (int)(blockDim.x >> 5) ? sb[lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_xor_sync(FULL, a, o);
+            b += __shfl_xor_sync(FULL, b, o);
+        }
+        if (lane == 0) { // float64 quotients are taken by one thread
+            sa[0] = a;
+            sb[0] = b / a;
+        }
+    }
+    __syncthreads();
+    a = sa[0];
+    b = sb[0];
+}
+
 // ---------------------------------------------------------------------------------------
 // Canonical averages from ln g (Eqs. 6-7): one CTA per temperature; u = <E>/N,
 // c = <(E - <E>)^2> / (N T^2), weights g(E) e^{-E/T} taken relative to one near their maximum.
@@ -1110,9 +1144,9 @@ namespace rewl {
 // result: a float32 pass finds the largest exponent and the bins within e^-82 of it (widened by a bound of
 // its own rounding error); only those, a tenth of the bins, take a quotient, an exponential and the
 // sums in float64.  Every bin does where float32 is too coarse to tell (large E/T), or where one bin holds
-// all the weight and c is made of the rest; the two largest exponents mostly tell, so that the second
-// pass is not taken for nothing first (Ising L=8, 500 frozen temperatures: 40 us before the selection, 45 with
-// it, 37 told beforehand).  Ising L=64, 500 temperatures: 393 us with a float64 quotient per bin in three
+// all the weight and c is made of the rest; the bins around that one mostly tell, so that the selected bins
+// are not summed for nothing first (Ising L=8, 500 frozen temperatures: 26 us before the selection, 32 with
+// it, 24 told beforehand).  Ising L=64, 500 temperatures: 393 us with a float64 quotient per bin in three
 // passes and two exponentials, 51 us.
 // ---------------------------------------------------------------------------------------
 constexpr int THERMO_THREADS = 256;
@@ -1123,7 +1157,7 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
                                                            double *__restrict__ Cv)
 {
     __shared__ double keep[THERMO_KEEP * THERMO_THREADS];
-    __shared__ float mx_s[32], next_s[32], big_s[32];
+    __shared__ float mx_s[32], big_s[32];
     __shared__ int arg_s[32];
     __shared__ double one_s; // float64 quotients are taken by one thread
     const double T = Ts[blockIdx.x];
@@ -1134,13 +1168,12 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     auto energy = [&](int b) { return model == 0 ? 4 * b - 2 * N : b - 2 * N; };
     auto coarse = [&](int b) { return __fmaf_rn(-(float)energy(b), invf, (float)lng[b]); };
-    // ---- float32: the largest exponent, its bin, the next largest, the largest |ln g|
-    float mx = -INFINITY, next = -INFINITY, big = 0.0f;
+    // ---- float32: the largest exponent, its bin, the largest |ln g|
+    float mx = -INFINITY, big = 0.0f;
     int arg = 0;
     for (int b = threadIdx.x; b <= B; b += blockDim.x) {
         const float l = (float)lng[b], x = __fmaf_rn(-(float)energy(b), invf, l);
         if (l > -INFINITY) big = fmaxf(big, fabsf(l));
-        next = fmaxf(next, fminf(mx, x));
         if (x > mx) {
             mx = x;
             arg = b;
@@ -1150,7 +1183,6 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     for (int o = 16; o > 0; o >>= 1) {
         const float om = __shfl_xor_sync(FULL, mx, o);
         const int oa = __shfl_xor_sync(FULL, arg, o);
-        next = fmaxf(fmaxf(next, __shfl_xor_sync(FULL, next, o)), fminf(mx, om));
         if (om > mx) {
             mx = om;
             arg = oa;
@@ -1159,13 +1191,11 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     }
     if (lane == 0) {
         mx_s[wid] = mx;
-        next_s[wid] = next;
         big_s[wid] = big;
         arg_s[wid] = arg;
     }
     __syncthreads();
     for (int i = 0; i < THERMO_THREADS / 32; ++i) { // the same choice in every thread
-        next = fmaxf(i == 0 ? next_s[0] : fmaxf(next, next_s[i]), i == 0 ? -INFINITY : fminf(mx, mx_s[i]));
         if (i == 0 || mx_s[i] > mx) {
             mx = mx_s[i];
             arg = arg_s[i];
@@ -1177,60 +1207,54 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     const float cut = mx - 82.0f - 2.0f * slack;
     // what the bins left out can add to s2 stays below its last bit where s2 >= enough s0
     const double enough = 1e17 * 2.5e-36 * (double)(B + 1) * 16.0 * (double)N * (double)N;
-    // one bin holds nearly all the weight: the others do not reach `enough`, so every bin is taken at once
-    // (either way is right; what this misses is found by s2 below)
-    const bool frozen = mx - next > 43.0f - __logf((float)(B + 1) * (float)N * (float)N);
+    // Where no bin beside the one of the largest exponent comes near it, the others will not reach `enough`, and
+    // every bin is taken at once.  A guess from the bins around it, and either way is right: s2 below tells.
+    const int beside = arg + (int)threadIdx.x - THERMO_THREADS / 2;
+    const bool frozen = !__syncthreads_or(beside >= 0 && beside <= B && beside != arg &&
+                                          coarse(beside) > mx - (43.0f - __logf((float)(B + 1) * (float)N * (float)N)));
     // energies from the bin of the largest exponent, so that a mean next to it keeps all its digits: c of a
     // frozen lattice is a sum over the other bins
     auto rel = [&](int b) { return (double)(energy(b) - energy(arg)); };
+    const double E0 = (double)energy(arg), l0 = lng[arg];
     double s0, e1, s2; // e1: relative mean
     for (bool all = frozen || !(slack < 8.0f && fabs(T) < INFINITY);; all = true) {
-        auto exponent = [&](int b) {
-            const double E = (double)energy(b);
-            if (all) return lng[b] - E / T;
-            const double q = E * inv; // E / T: one correction of E * (1 / T)
-            return lng[b] - __fma_rn(__fma_rn(-q, T, E), inv, q);
-        };
-        double ref;
+        double ref = -INFINITY; // largest exponent
         if (all) {
-            ref = -INFINITY;
             for (int b = threadIdx.x; b <= B; b += blockDim.x)
-                if (lng[b] > -INFINITY) ref = fmax(ref, exponent(b));
+                if (lng[b] > -INFINITY) ref = fmax(ref, lng[b] - (double)energy(b) / T);
             ref = block_reduce_max(ref);
-        } else {
-            ref = exponent(arg);
         }
+        auto weight = [&](int b, double R) { // of bin b, R = rel(b): relative to ref, or to bin `arg`
+            if (all) return exp((lng[b] - (E0 + R) / T) - ref);
+            const double q = R * inv; // R / T: one correction of R * (1 / T)
+            return exp((lng[b] - l0) - __fma_rn(__fma_rn(-q, T, R), inv, q));
+        };
         auto counts = [&](int b) { return all ? lng[b] > -INFINITY : coarse(b) > cut; };
-        double s1 = 0.0;
-        s0 = 0.0;
+        s0 = e1 = 0.0;
         int n = 0;
         for (int b = threadIdx.x; b <= B; b += blockDim.x)
             if (counts(b)) {
-                const double w = exp(exponent(b) - ref);
+                const double R = rel(b), w = weight(b, R);
                 if (n < THERMO_KEEP) keep[n * THERMO_THREADS + threadIdx.x] = w;
                 ++n;
                 s0 += w;
-                s1 += w * rel(b);
+                e1 += w * R;
             }
-        s0 = block_reduce_sum(s0);
-        s1 = block_reduce_sum(s1);
-        if (threadIdx.x == 0) one_s = s1 / s0;
-        __syncthreads();
-        e1 = one_s;
+        block_mean(s0, e1);
         s2 = 0.0;
         n = 0;
         for (int b = threadIdx.x; b <= B; b += blockDim.x)
             if (counts(b)) {
-                const double w = n < THERMO_KEEP ? keep[n * THERMO_THREADS + threadIdx.x] : exp(exponent(b) - ref);
+                const double R = rel(b), de = R - e1;
+                const double w = n < THERMO_KEEP ? keep[n * THERMO_THREADS + threadIdx.x] : weight(b, R);
                 ++n;
-                const double de = rel(b) - e1;
                 s2 += w * de * de;
             }
         s2 = block_reduce_sum(s2);
         if (all || s2 >= enough * s0) break; // else nearly one bin alone (low T): again with every bin
     }
     if (threadIdx.x == 0) {
-        U[blockIdx.x] = (energy(arg) + e1) / N;
+        U[blockIdx.x] = (E0 + e1) / N;
         Cv[blockIdx.x] = s2 / s0 / ((double)N * T * T);
     }
 }
