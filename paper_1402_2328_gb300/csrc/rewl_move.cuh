@@ -84,8 +84,8 @@ __device__ __forceinline__ int propose_dk(const int8_t *sp, const Lattice &lat, 
 // warp slots free (move kernel, Ising L=64 32 x 16, ln f = 2^-20: 378 us with the drawing in the
 // same warp, 259 us with a second one; 600 us with the 32-step chain of shuffles, match_any and
 // predicates before).  Workloads, us per launch of 10^4 moves, that kernel -> this one: Ising L=64 32 x 16
-// at 2^-20 600 -> 259, Ising L=32 8 x 8 at 2^-12 770 -> 332, Potts L=40 64 x 16 at 2^-10 810 -> 473,
-// Potts L=80 64 x 16 at 2^-24 700 -> 333, at ln f = 1 730 -> 584, Ising L=8 4 x 1 1960 -> 911.
+// at 2^-20 600 -> 259, Ising L=32 8 x 8 at 2^-12 770 -> 327, Potts L=40 64 x 16 at 2^-10 810 -> 470,
+// Potts L=80 64 x 16 at 2^-24 700 -> 336, at ln f = 1 730 -> 592, Ising L=8 4 x 1 1960 -> 902.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ double shadow_error(double maxabs, int T, double lnf, bool frozen)
 {
