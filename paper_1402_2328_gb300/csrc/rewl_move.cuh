@@ -84,8 +84,8 @@ __device__ __forceinline__ int propose_dk(const int8_t *sp, const Lattice &lat, 
 // warp slots free (move kernel, Ising L=64 32 x 16, ln f = 2^-20: 378 us with the drawing in the
 // same warp, 259 us with a second one; 600 us with the 32-step chain of shuffles, match_any and
 // predicates before).  Workloads, us per launch of 10^4 moves, that kernel -> this one: Ising L=64 32 x 16
-// at 2^-20 600 -> 259, Ising L=32 8 x 8 at 2^-12 770 -> 327, Potts L=40 64 x 16 at 2^-10 810 -> 470,
-// Potts L=80 64 x 16 at 2^-24 700 -> 336, at ln f = 1 730 -> 592, Ising L=8 4 x 1 1960 -> 902.
+// at 2^-20 600 -> 259, Ising L=32 8 x 8 at 2^-12 770 -> 327, Potts L=40 64 x 16 at 2^-10 810 -> 463,
+// Potts L=80 64 x 16 at 2^-24 700 -> 333, at ln f = 1 730 -> 580, Ising L=8 4 x 1 1960 -> 902.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ double shadow_error(double maxabs, int T, double lnf, bool frozen)
 {
@@ -357,7 +357,12 @@ __device__ __forceinline__ int agreed(int v) { return (int)__reduce_min_sync(FUL
 // Polls of shared memory before a warp gives up on its partner: the first warp on the second, which
 // is never long, and the second, asleep between polls, on the first, which may rebuild float64
 // values for seconds (a tie in every addition of a bin's 10^8 visits).
-constexpr int SPIN_LIMIT = 1 << 22, SLEEP_LIMIT = 1 << 28;
+constexpr int SPIN_LIMIT = 1 << 22, SLEEP_LIMIT = 1 << 25;
+// Sleep between the drawing warp's polls.  A ring in use holds 1.5 us of late steps or more beyond the block it has
+// no room for yet, so the walker does not wait for a sleeper, whose polls take issue slots.  us per launch at
+// 50 / 400 / 1200 ns: Potts L=80 64 x 16 at ln f = 1 593 / 580 / 572, at 2^-24 336 / 333 / 353, Potts L=40
+// 64 x 16 470 / 463 / 466, Ising L=64 32 x 16 at 2^-20 259 / 259 / 285.
+constexpr unsigned DRAW_SLEEP_NS = 400;
 
 // The second warp of a walker: draws blocks ahead of the first as the ring has room.
 template <bool ISING>
@@ -373,7 +378,7 @@ __device__ __forceinline__ void draw_walker(const State &s, const MoveCfg &c, co
     for (int g = 0; g < c.T + 64; g += 32) { // the first warp asks for 33 steps beyond the last
         for (int it = 0; g + 32 - agreed(load_acquire(mem.ctl + 1)) > MOVE_RING; ++it) {
             if (__any_sync(FULL, load_acquire(mem.ctl + 2) != 0) || it > SLEEP_LIMIT) return;
-            __nanosleep(50);
+            __nanosleep(DRAW_SLEEP_NS);
         }
         draw_block<ISING, false>(s, c, mem, slot, st0, g, before, lane);
         __syncwarp();
