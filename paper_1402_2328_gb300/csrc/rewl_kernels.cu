@@ -1144,20 +1144,21 @@ __device__ __forceinline__ void block_mean(double &a, double &b)
 // result: a float32 pass finds the largest exponent and the bins within e^-82 of it (widened by a bound of
 // its own rounding error); only those, a tenth of the bins, take a quotient, an exponential and the
 // sums in float64.  Every bin does where float32 is too coarse to tell (large E/T), or where one bin holds
-// all the weight and c is made of the rest; the bins around that one mostly tell, so that the selected bins
-// are not summed for nothing first (Ising L=8, 500 frozen temperatures: 26 us before the selection, 32 with
-// it, 24 told beforehand).  Ising L=64, 500 temperatures: 393 us with a float64 quotient per bin in three
+// all the weight and c is made of the rest; the largest exponents of the threads mostly tell, so that the
+// selected bins are not summed for nothing first (Ising L=8, 500 frozen temperatures: 26 us before the
+// selection, 32 with it, 24 told beforehand).  Four CTAs an SM: left to itself the compiler takes 48
+// registers and spills (54 us).  Ising L=64, 500 temperatures: 393 us with a float64 quotient per bin in three
 // passes and two exponentials, 51 us.
 // ---------------------------------------------------------------------------------------
 constexpr int THERMO_THREADS = 256;
 constexpr int THERMO_KEEP = 8; // weights a thread keeps between the two sums
 
-__global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restrict__ lng, int B, int model, int N,
-                                                           const double *__restrict__ Ts, double *__restrict__ U,
-                                                           double *__restrict__ Cv)
+__global__ void __launch_bounds__(THERMO_THREADS, 4)
+    k_thermo(const double *__restrict__ lng, int B, int model, int N, const double *__restrict__ Ts,
+             double *__restrict__ U, double *__restrict__ Cv)
 {
     __shared__ double keep[THERMO_KEEP * THERMO_THREADS];
-    __shared__ float mx_s[32], big_s[32];
+    __shared__ float mx_s[32], next_s[32], big_s[32];
     __shared__ int arg_s[32];
     __shared__ double one_s; // float64 quotients are taken by one thread
     const double T = Ts[blockIdx.x];
@@ -1168,8 +1169,8 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     auto energy = [&](int b) { return model == 0 ? 4 * b - 2 * N : b - 2 * N; };
     auto coarse = [&](int b) { return __fmaf_rn(-(float)energy(b), invf, (float)lng[b]); };
-    // ---- float32: the largest exponent, its bin, the largest |ln g|
-    float mx = -INFINITY, big = 0.0f;
+    // ---- float32: the largest exponent, its bin, the largest of the other threads', the largest |ln g|
+    float mx = -INFINITY, next = -INFINITY, big = 0.0f;
     int arg = 0;
     for (int b = threadIdx.x; b <= B; b += blockDim.x) {
         const float l = (float)lng[b], x = __fmaf_rn(-(float)energy(b), invf, l);
@@ -1183,6 +1184,7 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     for (int o = 16; o > 0; o >>= 1) {
         const float om = __shfl_xor_sync(FULL, mx, o);
         const int oa = __shfl_xor_sync(FULL, arg, o);
+        next = fmaxf(fmaxf(next, __shfl_xor_sync(FULL, next, o)), fminf(mx, om));
         if (om > mx) {
             mx = om;
             arg = oa;
@@ -1191,11 +1193,13 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     }
     if (lane == 0) {
         mx_s[wid] = mx;
+        next_s[wid] = next;
         big_s[wid] = big;
         arg_s[wid] = arg;
     }
     __syncthreads();
     for (int i = 0; i < THERMO_THREADS / 32; ++i) { // the same choice in every thread
+        next = i == 0 ? next_s[0] : fmaxf(fmaxf(next, next_s[i]), fminf(mx, mx_s[i]));
         if (i == 0 || mx_s[i] > mx) {
             mx = mx_s[i];
             arg = arg_s[i];
@@ -1208,27 +1212,30 @@ __global__ void __launch_bounds__(THERMO_THREADS) k_thermo(const double *__restr
     // what the bins left out can add to s2 stays below its last bit where s2 >= enough s0
     const double enough = 1e17 * 2.5e-36 * (double)(B + 1) * 16.0 * (double)N * (double)N;
     // Where no bin beside the one of the largest exponent comes near it, the others will not reach `enough`, and
-    // every bin is taken at once.  A guess from the bins around it, and either way is right: s2 below tells.
-    const int beside = arg + (int)threadIdx.x - THERMO_THREADS / 2;
-    const bool frozen = !__syncthreads_or(beside >= 0 && beside <= B && beside != arg &&
-                                          coarse(beside) > mx - (43.0f - __logf((float)(B + 1) * (float)N * (float)N)));
-    // energies from the bin of the largest exponent, so that a mean next to it keeps all its digits: c of a
-    // frozen lattice is a sum over the other bins
-    auto rel = [&](int b) { return (double)(energy(b) - energy(arg)); };
-    const double E0 = (double)energy(arg), l0 = lng[arg];
-    double s0, e1, s2; // e1: relative mean
+    // every bin is taken at once.  Either way is right: s2 below tells.
+    const bool frozen = mx - next > 43.0f - __logf((float)(B + 1) * (float)N * (float)N);
+    double s0, e1, s2, E0; // e1: mean energy from E0
     for (bool all = frozen || !(slack < 8.0f && fabs(T) < INFINITY);; all = true) {
-        double ref = -INFINITY; // largest exponent
-        if (all) {
-            for (int b = threadIdx.x; b <= B; b += blockDim.x)
-                if (lng[b] > -INFINITY) ref = fmax(ref, lng[b] - (double)energy(b) / T);
-            ref = block_reduce_max(ref);
-        }
-        auto weight = [&](int b, double R) { // of bin b, R = rel(b): relative to ref, or to bin `arg`
-            if (all) return exp((lng[b] - (E0 + R) / T) - ref);
-            const double q = R * inv; // R / T: one correction of R * (1 / T)
-            return exp((lng[b] - l0) - __fma_rn(__fma_rn(-q, T, R), inv, q));
+        // every bin: energies from the bin of the largest exponent, so that a mean next to it keeps all its
+        // digits, as c of a frozen lattice is a sum over the other bins
+        const int e0 = all ? energy(arg) : 0;
+        E0 = (double)e0;
+        auto rel = [&](int b) { return (double)(energy(b) - e0); };
+        auto exponent = [&](double R) { // of the bin at energy E0 + R, its ln g aside
+            if (all) return (E0 + R) / T;
+            const double q = R * inv; // E / T: one correction of E * (1 / T)
+            return __fma_rn(__fma_rn(-q, T, R), inv, q);
         };
+        double ref;
+        if (all) {
+            ref = -INFINITY;
+            for (int b = threadIdx.x; b <= B; b += blockDim.x)
+                if (lng[b] > -INFINITY) ref = fmax(ref, lng[b] - exponent(rel(b)));
+            ref = block_reduce_max(ref);
+        } else {
+            ref = lng[arg] - exponent(rel(arg));
+        }
+        auto weight = [&](int b, double R) { return exp((lng[b] - exponent(R)) - ref); };
         auto counts = [&](int b) { return all ? lng[b] > -INFINITY : coarse(b) > cut; };
         s0 = e1 = 0.0;
         int n = 0;
