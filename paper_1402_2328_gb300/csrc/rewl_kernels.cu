@@ -370,8 +370,6 @@ __device__ __forceinline__ void check_window(const State &s, const int w, const 
     }
 }
 
-// Replica exchange (Eq. 1) between windows (w, w+1), w = round mod 2.  One warp per pair; the
-// swap itself exchanges configuration indices and bins.
 // Partner permutation of the exchange of pair (gw, gw+1) in round rd (global window index gw):
 // Fisher-Yates from Philox draws (i, rd, gw, swap tag), i = m-1 .. 1.  One warp; perm in shared
 // memory, valid after the call for every lane.
@@ -407,9 +405,9 @@ __device__ __forceinline__ bool exchange_accept(const State &s, int gw, long lon
     return lnu64(r.x) < lnP;
 }
 
-// The exchange of windows (w, w+1) in round rd, by one warp: the permutation's random draws and the
-// m decisions are lane-parallel (each decision touches its own two walker slots); only the
-// Fisher-Yates swaps themselves run in order.  Other CTAs of the launch wrote some of what is read
+// Replica exchange (Eq. 1) of windows (w, w+1), w of the parity of round rd, by one warp: configuration
+// indices and bins change places.  The permutation's random draws and the m decisions are lane-parallel
+// (each decision touches its own two walker slots); only the Fisher-Yates swaps themselves run in order.  Other CTAs of the launch wrote some of what is read
 // here, so loads go past the L1.
 __device__ __forceinline__ void swap_windows(const State &s, const int w, const long long rd)
 {
