@@ -407,8 +407,8 @@ __device__ __forceinline__ bool exchange_accept(const State &s, int gw, long lon
 
 // Replica exchange (Eq. 1) of windows (w, w+1), w of the parity of round rd, by one warp: configuration
 // indices and bins change places.  The permutation's random draws and the m decisions are lane-parallel
-// (each decision touches its own two walker slots); only the Fisher-Yates swaps themselves run in order.  Other CTAs of the launch wrote some of what is read
-// here, so loads go past the L1.
+// (each decision touches its own two walker slots); only the Fisher-Yates swaps themselves run in order.
+// Other CTAs of the launch wrote some of what is read here, so loads go past the L1.
 __device__ __forceinline__ void swap_windows(const State &s, const int w, const long long rd)
 {
     const int lane = threadIdx.x & 31;
